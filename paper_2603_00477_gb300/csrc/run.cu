@@ -6,6 +6,7 @@
 // `out` and the workspace so that the last sweep lands in `out`; `in` is
 // never written.  The fixed halo of `in` is copied once to every buffer
 // that a sweep writes, because sweeps only write interior points.
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -15,32 +16,73 @@ namespace gbs {
 
 namespace {
 
-template <typename T>
-__global__ void halo_copy_kernel(const T *__restrict__ in, T *__restrict__ out, T *__restrict__ out2, int64_t Ez,
-                                 int64_t Ey, int64_t Ex, int R, int zhalo)
+// The stored grid as rows (z, y) of Ex cells.  Halo rows are copied whole and
+// interior rows only at their R cells on each end.  Blocks [0, seg_blocks)
+// take the halo rows, cut into segments of kHaloSeg cells, one warp per
+// segment; the other blocks take the interior rows' ends, one thread per
+// cell.  The copy is a few hundred KB to a few MB with no reuse: it is bound
+// by memory latency, so the work is spread until every thread moves a handful
+// of cells.  One warp per whole halo row made a 16384-cell row a serial chain
+// of 512 loads: 77 us on a 16384^2 FP32 grid (10 us on 1021 x 1531) against
+// 5 us (3 us) now.
+constexpr int kHaloSeg = 512;   // cells of a halo-row segment (16 per lane)
+constexpr int kHaloThreads = 256;
+
+// Halo row j (0 .. count-1) as a stored row index: in 3-D the R first and R
+// last planes whole, then the 2R edge rows of each interior plane.
+__device__ __forceinline__ int64_t halo_row(int64_t j, int64_t Ez, int64_t Ey, int R, int zhalo)
 {
-    // one warp per stored row (z, y); halo rows are copied whole, interior
-    // rows only at their R cells on each end
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < Ez * Ey; row += warps) {
-        const int64_t z = row / Ey, y = row % Ey;
-        const bool halo_row = y < R || y >= Ey - R || (zhalo && (z < R || z >= Ez - R));
-        const int64_t base = row * Ex;
-        if (halo_row) {
-            for (int64_t x = lane; x < Ex; x += 32) {
-                T v = in[base + x];
-                out[base + x] = v;
-                if (out2) out2[base + x] = v;
+    int64_t z0 = 0;
+    if (zhalo) {
+        const int64_t nplane = 2 * (int64_t)R * Ey;
+        if (j < nplane) {
+            const int64_t z = j / Ey;
+            return (z < R ? z : Ez - 2 * R + z) * Ey + j % Ey;
+        }
+        j -= nplane;
+        z0 = R;
+    }
+    const int64_t z = z0 + j / (2 * R), i = j % (2 * R);
+    return z * Ey + (i < R ? i : Ey - 2 * R + i);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kHaloThreads)
+    halo_copy_kernel(const T *__restrict__ in, T *__restrict__ out, T *__restrict__ out2, int64_t Ez, int64_t Ey,
+                     int64_t Ex, int R, int zhalo, int64_t nsegs, unsigned seg_blocks)
+{
+    if (blockIdx.x < seg_blocks) {
+        const int lane = threadIdx.x & 31;
+        const int64_t per_row = (Ex + kHaloSeg - 1) / kHaloSeg, warps = (int64_t)seg_blocks * (kHaloThreads / 32);
+        for (int64_t s = (int64_t)blockIdx.x * (kHaloThreads / 32) + (threadIdx.x >> 5); s < nsegs; s += warps) {
+            const int64_t base = halo_row(s / per_row, Ez, Ey, R, zhalo) * Ex, x0 = (s % per_row) * kHaloSeg;
+            T v[kHaloSeg / 32];
+#pragma unroll
+            for (int i = 0; i < kHaloSeg / 32; ++i) {
+                const int64_t x = x0 + lane + 32 * i;
+                if (x < Ex) v[i] = in[base + x];
             }
-        } else {
-            for (int64_t i = lane; i < 2 * R; i += 32) {
-                const int64_t x = i < R ? i : Ex - 2 * R + i;
-                T v = in[base + x];
-                out[base + x] = v;
-                if (out2) out2[base + x] = v;
+#pragma unroll
+            for (int i = 0; i < kHaloSeg / 32; ++i) {
+                const int64_t x = x0 + lane + 32 * i;
+                if (x < Ex) {
+                    out[base + x] = v[i];
+                    if (out2) out2[base + x] = v[i];
+                }
             }
         }
+        return;
+    }
+    // interior row q = (plane, row), its cell i of 2R (R left, R right)
+    const int64_t niy = Ey - 2 * R, n = (zhalo ? Ez - 2 * R : Ez) * niy * 2 * R;
+    const int64_t stride = (int64_t)(gridDim.x - seg_blocks) * kHaloThreads;
+    for (int64_t e = (int64_t)(blockIdx.x - seg_blocks) * kHaloThreads + threadIdx.x; e < n; e += stride) {
+        const int64_t q = e / (2 * R), i = e % (2 * R);
+        const int64_t z = q / niy + (zhalo ? R : 0), y = q % niy + R;
+        const int64_t a = (z * Ey + y) * Ex + (i < R ? i : Ex - 2 * R + i);
+        const T v = in[a];
+        out[a] = v;
+        if (out2) out2[a] = v;
     }
 }
 
@@ -48,18 +90,22 @@ __global__ void halo_copy_kernel(const T *__restrict__ in, T *__restrict__ out, 
 
 stencil_status launch_halo_copy(const Plan &p, const void *in, void *out, void *out2, cudaStream_t st)
 {
-    const int R = p.pat.r;
-    const int64_t rows = p.ext[0] * p.ext[1];
-    int64_t blocks = (rows + 7) / 8;
-    if (blocks > 152 * 16) blocks = 152 * 16;
+    const int R = p.pat.r, zhalo = p.pat.d == 3;
+    const int64_t Ez = p.ext[0], Ey = p.ext[1], Ex = p.ext[2];
+    const int64_t nz = zhalo ? Ez - 2 * R : Ez;
+    const int64_t nhalo = (zhalo ? 2 * (int64_t)R * Ey : 0) + nz * 2 * R;
+    const int64_t nsegs = nhalo * ((Ex + kHaloSeg - 1) / kHaloSeg);
+    const int64_t cells = nz * (Ey - 2 * R) * 2 * R;
+    // at most 16 blocks per SM for each part; the kernel's loops cover the rest
+    auto cap = [](int64_t b) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, 152 * 16)); };
+    const unsigned seg_blocks = cap((nsegs + kHaloThreads / 32 - 1) / (kHaloThreads / 32));
+    const unsigned blocks = seg_blocks + cap((cells + kHaloThreads - 1) / kHaloThreads);
     if (p.dtype == STENCIL_F64)
-        halo_copy_kernel<double><<<(unsigned)blocks, 256, 0, st>>>((const double *)in, (double *)out,
-                                                                   (double *)out2, p.ext[0], p.ext[1], p.ext[2],
-                                                                   R, p.pat.d == 3);
+        halo_copy_kernel<double><<<blocks, kHaloThreads, 0, st>>>((const double *)in, (double *)out, (double *)out2,
+                                                                  Ez, Ey, Ex, R, zhalo, nsegs, seg_blocks);
     else
-        halo_copy_kernel<float><<<(unsigned)blocks, 256, 0, st>>>((const float *)in, (float *)out, (float *)out2,
-                                                                  p.ext[0], p.ext[1], p.ext[2], R,
-                                                                  p.pat.d == 3);
+        halo_copy_kernel<float><<<blocks, kHaloThreads, 0, st>>>((const float *)in, (float *)out, (float *)out2, Ez,
+                                                                 Ey, Ex, R, zhalo, nsegs, seg_blocks);
     note_launch();
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "halo_copy launch");
