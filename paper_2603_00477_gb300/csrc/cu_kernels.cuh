@@ -72,39 +72,12 @@ struct Weights {
 // ---------------------------------------------------------------------------
 // 2-D: tile BY x BX, strips of V rows.
 // ---------------------------------------------------------------------------
-// Band mode (band > 0): only the tiles of the ring of tile rows/columns that
-// touch the band run (a 1-D grid, ring.count blocks), and only points closer
-// than `band` to the interior boundary are written.  Used after a
-// tensor-core sweep, whose fused kernel is exact only away from the
-// boundary.
-struct Ring {
-    int band;        // 0: every tile, row-major over ntx columns
-    int nty, ntx;    // tiles along y and x
-    int rows_tb;     // tile rows taken whole: min(nty, top_w + bottom rows)
-    int top_w;       // tile rows touching the top band
-    int cols_lr;     // tile columns taken in the other rows: min(ntx, left_w + right cols)
-    int left_w;      // tile columns touching the left band
-    int xshift;      // band 0, FP32: the tile grid starts xshift columns further left so that
-                     // every staged window begins on a 16-byte boundary (then vec16 = 1)
+struct Tiles {
+    int ntx;         // tiles along x (row-major tile order)
+    int xshift;      // FP32: the tile grid starts xshift columns further left so that every
+                     // staged window begins on a 16-byte boundary (then vec16 = 1)
     int vec16;       // stage interior tiles with 16-byte copies
 };
-
-// Tile id -> (tile row, tile column): first the whole tile rows (the top_w
-// top ones, then the bottom ones), then, row by row, the left and right tile
-// columns of the remaining rows.
-__device__ __forceinline__ void ring_tile(const Ring &g, int id, int *by, int *bx)
-{
-    if (id < g.rows_tb * g.ntx) {
-        const int rr = id / g.ntx;
-        *bx = id % g.ntx;
-        *by = rr < g.top_w ? rr : g.nty - g.rows_tb + rr;
-    } else {
-        const int id2 = id - g.rows_tb * g.ntx;
-        const int cc = id2 % g.cols_lr;
-        *by = g.top_w + id2 / g.cols_lr;
-        *bx = cc < g.left_w ? cc : g.ntx - g.cols_lr + cc;
-    }
-}
 
 // Asynchronous global -> shared copy of one element (cp.async, L1-allocating);
 // src_bytes = 0 writes zeros without reading global memory.
@@ -291,7 +264,7 @@ template <int SHAPE, int R, int D, typename WT>
 __device__ __forceinline__ void f32_substep4(const float *__restrict__ src, float *__restrict__ dst,
                                              float *__restrict__ out, const WT &wt, int P, int lo, int hiY, int hiX,
                                              int64_t Y0, int64_t X0, int64_t Ey, int64_t Ex, bool last,
-                                             bool all_interior, int band)
+                                             bool all_interior)
 {
     constexpr int NS = 2 * R + 1;          // rotating slots
     constexpr int NV = 2 * R + 4 + D;      // window values per row
@@ -301,8 +274,7 @@ __device__ __forceinline__ void f32_substep4(const float *__restrict__ src, floa
     // enough strips to give every thread a work item, each of >= 4 rows
     const int nstrips = max(1, min(max(1, ch / 4), (int)((blockDim.x + nquads - 1) / nquads)));
     const int S = (ch + nstrips - 1) / nstrips;
-    const int64_t ny = Ey - 2 * R, nx = Ex - 2 * R;
-    const bool fast = all_interior && band == 0;
+    const bool fast = all_interior;
 
     for (int item = threadIdx.x; item < nstrips * nquads; item += blockDim.x) {
         const int sy = item / nquads, qx = item - sy * nquads;
@@ -339,12 +311,7 @@ __device__ __forceinline__ void f32_substep4(const float *__restrict__ src, floa
                 const int64_t gx = X0 + x + h;
                 const bool interior = rowint && gx >= R && gx < Ex - R;
                 if (last) {
-                    bool keep = interior;
-                    if (band > 0) {
-                        const int64_t iy = gy - R, ix = gx - R;
-                        keep = keep && (iy < band || ix < band || ny - 1 - iy < band || nx - 1 - ix < band);
-                    }
-                    if (keep) out[gy * Ex + gx] = a[h];
+                    if (interior) out[gy * Ex + gx] = a[h];
                 } else {
                     dst[y * P + x + h] = interior ? a[h] : src[y * P + x + h];
                 }
@@ -544,7 +511,7 @@ template <typename T, int SHAPE, int R, int V>
 __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
     cu2d_sweep(const T *__restrict__ in, T *__restrict__ out,
                const __grid_constant__ Weights<T, Taps<SHAPE, 2, R>::K> wt, int64_t Ey, int64_t Ex, int BY, int BX,
-               int t, const Ring ring, int ntiles)
+               int t, const Tiles tiles, int ntiles)
 {
     constexpr int KT = Taps<SHAPE, 2, R>::K;
     constexpr bool kSmemW = sizeof(T) == 8;
@@ -558,26 +525,21 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
     const size_t buf = buf_elems<T>(H, W);
     T *const stage0 = reinterpret_cast<T *>(base), *const stage1 = stage0 + buf;
     T *work = reinterpret_cast<T *>(base) + 2 * buf;
-    const int64_t ny = Ey - 2 * R, nx = Ex - 2 * R;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
 
     auto origin = [&](int id, int64_t *Y0, int64_t *X0) {
         int by, bx;
-        if (ring.band > 0) {
-            ring_tile(ring, id, &by, &bx);
-        } else {
-            by = id / ring.ntx;
-            bx = id % ring.ntx;
-        }
+        by = id / tiles.ntx;
+        bx = id % tiles.ntx;
         *Y0 = R + (int64_t)by * BY - (int64_t)t * R;
-        *X0 = R + (int64_t)bx * BX - (int64_t)t * R - ring.xshift;
+        *X0 = R + (int64_t)bx * BX - (int64_t)t * R - tiles.xshift;
     };
     // Stage the dependency region of a tile; cells outside the stored array
     // are zero-filled and never used by an interior point.
     auto prefetch = [&](int id, T *dst) {
         int64_t Y0, X0;
         origin(id, &Y0, &X0);
-        if (sizeof(T) == 4 && ring.vec16 && Y0 >= 0 && X0 >= 0 && Y0 + H <= Ey && X0 + P <= Ex) {
+        if (sizeof(T) == 4 && tiles.vec16 && Y0 >= 0 && X0 >= 0 && Y0 + H <= Ey && X0 + P <= Ex) {
             // 16-byte copies: X0, the row length and the input are 16-byte aligned
             const T *g = in + Y0 * Ex + X0;
             for (int y = warp; y < H; y += nwarps) {
@@ -630,7 +592,7 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
             if constexpr (sizeof(T) == 4) {
                 const bool all_int = Y0 + lo >= R && Y0 + hiY <= Ey - R && X0 + lo >= R && X0 + hiX <= Ex - R;
                 if constexpr (R <= 2) {
-                    if (all_int && ring.band == 0 && (cw & 3) == 0 && ch >= 8) {
+                    if (all_int && (cw & 3) == 0 && ch >= 8) {
                         // strips of 8 rows, or of 4 when that tiles the region exactly
                         const bool s4 = (ch & 7) != 0 && (ch & 3) == 0;
                         f32_fixed_dispatch<SHAPE, R>((lo - R) & 3, s4, src, dst, out, wt, P, lo, hiY, hiX, Y0, X0,
@@ -645,7 +607,7 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
                     // larger radii: strips of 2 rows (each item reads 2 + 2R rows
                     // for 8 outputs: loads stay a few % of the (2R+1)^2 taps, and
                     // the unrolled code stays a few thousand FMAs)
-                    if (all_int && ring.band == 0 && (cw & 3) == 0 && ch >= 2) {
+                    if (all_int && (cw & 3) == 0 && ch >= 2) {
                         f32_fixed_dispatch2<SHAPE, R>((lo - R) & 3, src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ex,
                                                       last);
                         __syncthreads();
@@ -657,20 +619,16 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
                 }
                 switch ((lo - R) & 3) {  // offset of the first window within its 16-byte chunk
                 case 0:
-                    f32_substep4<SHAPE, R, 0>(src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ey, Ex, last, all_int,
-                                              ring.band);
+                    f32_substep4<SHAPE, R, 0>(src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ey, Ex, last, all_int);
                     break;
                 case 1:
-                    f32_substep4<SHAPE, R, 1>(src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ey, Ex, last, all_int,
-                                              ring.band);
+                    f32_substep4<SHAPE, R, 1>(src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ey, Ex, last, all_int);
                     break;
                 case 2:
-                    f32_substep4<SHAPE, R, 2>(src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ey, Ex, last, all_int,
-                                              ring.band);
+                    f32_substep4<SHAPE, R, 2>(src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ey, Ex, last, all_int);
                     break;
                 default:
-                    f32_substep4<SHAPE, R, 3>(src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ey, Ex, last, all_int,
-                                              ring.band);
+                    f32_substep4<SHAPE, R, 3>(src, dst, out, wt, P, lo, hiY, hiX, Y0, X0, Ey, Ex, last, all_int);
                     break;
                 }
                 __syncthreads();
@@ -715,13 +673,7 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
                         const int64_t gy = Y0 + y;
                         const bool interior = colint && gy >= R && gy < Ey - R;
                         if (last) {
-                            bool keep = interior;
-                            if (ring.band > 0) {
-                                const int64_t iy = gy - R, ix = gx - R;
-                                keep = keep && (iy < ring.band || ix < ring.band || ny - 1 - iy < ring.band ||
-                                                nx - 1 - ix < ring.band);
-                            }
-                            if (keep) out[gy * Ex + gx] = acc[j];
+                            if (interior) out[gy * Ex + gx] = acc[j];
                         } else {
                             dst[y * P + x] = interior ? acc[j] : src[y * P + x];
                         }

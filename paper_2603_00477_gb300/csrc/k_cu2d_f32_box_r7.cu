@@ -3,9 +3,9 @@
 
 namespace gbs {
 
-stencil_status launch_cu2d_f32_box_r7(const Plan &p, const void *in, void *out, int t, int band, cudaStream_t st)
+stencil_status launch_cu2d_f32_box_r7(const Plan &p, const void *in, void *out, int t, cudaStream_t st)
 {
-    return cuimpl::launch2d_range<float, 0, 7, 7>(p, in, out, t, band, st);
+    return cuimpl::launch2d_range<float, 0, 7, 7>(p, in, out, t, st);
 }
 
 }  // namespace gbs

@@ -3,10 +3,10 @@
 
 namespace gbs {
 
-stencil_status launch_cu2d_f64(const Plan &p, const void *in, void *out, int t, int band, cudaStream_t st)
+stencil_status launch_cu2d_f64(const Plan &p, const void *in, void *out, int t, cudaStream_t st)
 {
-    if (p.pat.shape == STENCIL_BOX) return cuimpl::launch2d_range<double, 0, 1, 7>(p, in, out, t, band, st);
-    return cuimpl::launch2d_range<double, 1, 1, 7>(p, in, out, t, band, st);
+    if (p.pat.shape == STENCIL_BOX) return cuimpl::launch2d_range<double, 0, 1, 7>(p, in, out, t, st);
+    return cuimpl::launch2d_range<double, 1, 1, 7>(p, in, out, t, st);
 }
 
 }  // namespace gbs

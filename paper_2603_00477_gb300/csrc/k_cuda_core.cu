@@ -67,22 +67,16 @@ stencil_status launch_cu_sweep(const Plan &p, const void *in, void *out, int t, 
 {
     if (p.pat.d == 3) return launch_cu3d(p, in, out, t, st);
     if (p.pat.d != 2) return fail(STENCIL_ERR_UNSUPPORTED, "no CUDA-core kernel for this d");
-    return launch_cu_band(p, in, out, t, 0, st);
-}
-
-stencil_status launch_cu_band(const Plan &p, const void *in, void *out, int t, int band, cudaStream_t st)
-{
-    if (p.pat.d != 2) return fail(STENCIL_ERR_UNSUPPORTED, "band sweep: 2-D only");
-    if (p.dtype == STENCIL_F64) return launch_cu2d_f64(p, in, out, t, band, st);
+    if (p.dtype == STENCIL_F64) return launch_cu2d_f64(p, in, out, t, st);
     const int r = p.pat.r;
     if (p.pat.shape == STENCIL_BOX) {
-        if (r <= 3) return launch_cu2d_f32_box_r13(p, in, out, t, band, st);
-        if (r <= 5) return launch_cu2d_f32_box_r45(p, in, out, t, band, st);
-        if (r == 6) return launch_cu2d_f32_box_r6(p, in, out, t, band, st);
-        return launch_cu2d_f32_box_r7(p, in, out, t, band, st);
+        if (r <= 3) return launch_cu2d_f32_box_r13(p, in, out, t, st);
+        if (r <= 5) return launch_cu2d_f32_box_r45(p, in, out, t, st);
+        if (r == 6) return launch_cu2d_f32_box_r6(p, in, out, t, st);
+        return launch_cu2d_f32_box_r7(p, in, out, t, st);
     }
-    if (r <= 4) return launch_cu2d_f32_star_r14(p, in, out, t, band, st);
-    return launch_cu2d_f32_star_r57(p, in, out, t, band, st);
+    if (r <= 4) return launch_cu2d_f32_star_r14(p, in, out, t, st);
+    return launch_cu2d_f32_star_r57(p, in, out, t, st);
 }
 
 }  // namespace gbs
