@@ -30,12 +30,10 @@ stencil_status launch_split_sweep(const Plan &p, const void *in, void *out, int 
 // Read and clear the split kernel's own error word (part of read_device_error).
 stencil_status read_split_error(int *flag);
 
-// One fused sweep of depth t of an FP32 grid on the FP16 / BF16 tensor cores
-// with wide MMAs (k_wide.cu; precision f16, f16x3 when split, bf16x3 when
-// split and bf16), without the band sweep.  STENCIL_ERR_UNSUPPORTED when its
-// operands do not fit (tc_wide_nrows == 0) or for BF16 without the split.
-stencil_status launch_wide_sweep(const Plan &p, const void *in, void *out, int t, bool split, bool bf16,
-                                 cudaStream_t st);
+// One fused sweep of depth t of a 2-D FP32 grid on the tcgen05 tensor cores
+// in the plan's precision form (k_wide.cu: tf32, tf32x3, f16, f16x3, bf16x3),
+// without the band sweep.  STENCIL_ERR_UNSUPPORTED for t*r > 12.
+stencil_status launch_wide_sweep(const Plan &p, const void *in, void *out, int t, cudaStream_t st);
 
 // Read and clear the wide kernel's own error word (part of read_device_error).
 stencil_status read_wide_error(int *flag);

@@ -488,8 +488,7 @@ static stencil_status enumerate(Plan *p, std::vector<Cand> *out)
                 } else {
                     c.tile[0] = 1;
                     c.tile[1] = p->dtype == STENCIL_F64 ? 64 : 128;
-                    c.tile[2] = p->dtype == STENCIL_F64 ? 64 : (prec == STENCIL_PREC_TF32 ? 64 : (prec == STENCIL_PREC_TF32X3 ? 32 : 64));
-                    if (path == STENCIL_PATH_SPARSE_TENSOR_CORE) c.tile[2] = 64;
+                    c.tile[2] = 64;
                     if (prec == STENCIL_PREC_OZAKI) {
                         c.tile[1] = 128;
                         c.tile[2] = 16 * split_nacc(t * r, slices);
@@ -497,12 +496,14 @@ static stencil_status enumerate(Plan *p, std::vector<Cand> *out)
                     if (d == 3) {
                         c.tile[1] = tc_wide3_nrows(shape, r);  // one plane: rows (MMA N) x 128 columns
                         c.tile[2] = 128;
-                    } else if (prec == STENCIL_PREC_BF16X3 || prec == STENCIL_PREC_F16 || prec == STENCIL_PREC_F16X3) {
-                        // the wide kernel: output rows (MMA N) x 128 columns
-                        const int nr = tc_wide_nrows(r, t, prec != STENCIL_PREC_F16);
-                        if (nr == 0) continue;  // t r > 12
-                        c.tile[1] = nr;
-                        c.tile[2] = 128;
+                    } else if (p->dtype == STENCIL_F32 && path == STENCIL_PATH_TENSOR_CORE) {
+                        // the block kernels (k_wide.cu): 16 gn output rows x 64 columns
+                        const bool tf = prec == STENCIL_PREC_TF32 || prec == STENCIL_PREC_TF32X3;
+                        const BlockTile bt = tc_block_tile(
+                            t * r, tf, prec != STENCIL_PREC_TF32 && prec != STENCIL_PREC_F16, p->dims[1], p->ext[2],
+                            device_sms());
+                        c.tile[1] = 16 * bt.gn;
+                        c.tile[2] = 64;
                     }
                     TcGeometry g = tc_geometry(shape, d, r, t, p->dtype, prec, path);
                     ModelOut m = model_eval(shape, d, r, t, D, g.sparsity, beta_of(prec, slices), P_cu,

@@ -85,59 +85,85 @@ inline int tc_ws_ntile(int shape, int r, int t, bool split)
     return 8;
 }
 
-// Wide FP16 kernel (tc2d_wide): the Toeplitz factor of line a is the A
-// operand over M = 128 output columns (stored in reverse order, so that
-// A[m'][k] depends on k + m' only) and K = 16 nkb window columns,
-// nkb = ceil((128 + 2R) / 16); the input tile is the B operand over N = nr
-// output rows.  Line a's A operand for every K block is read from one strip
-// of 2 nkb + 15 core matrices (128 bytes each), non-zero only in core
-// matrices 15 .. (127 + 2R) / 8, so consecutive lines' strips are placed
-// max(2 nkb, (127 + 2R) / 8 + 1) core matrices apart and overlap in zeros.
-struct WideGeom {
-    int nkb, strip_len, delta, hs, nbuf;
-    size_t strip_bytes, in_bytes, smem;
+// Line form of the FP16 / BF16 precisions: the Toeplitz factor of line a over
+// 128 output columns (stored in reverse order, A[m'][k] depends on k + m' only)
+// and the window of 128 + 2R columns in K blocks of 16.  This is the layout
+// stencil_plan_tc_layout exports and the sparsity S and the model of these
+// precisions refer to (every R <= kWideMaxR has one); rows per tile as the
+// operands of that form fit in 227 KB.  The 2-D kernels issue the denser block
+// form below; the 3-D kernel (tc3d_wide) issues the line form.
+constexpr int kWideMaxR = 12;
+
+inline int tc_wide_nrows(int r, int t, bool split)
+{
+    const int R = t * r;
+    if (R > kWideMaxR) return 0;
+    return !split && R <= 9 ? 256 : 128;
+}
+
+// Block form of the 2-D kernels (k_wide.cu): MMA rows = the 16 x 8 outputs of a
+// block, MMA columns = 8 gn block positions (8 across, gn down), K = the
+// 16-byte chunks of the block's (16 + 2R) x (8 + 2R) neighbourhood.
+struct BlockTile {
+    int gn = 0;    // block rows: the tile is 16 gn x 64 outputs (0: no tile)
+    int nbuf = 0;  // operand buffers
+    int nc = 0;    // 16-byte chunks of a neighbourhood row
+    int pc = 0;    // 8-column units of a staged row
+    int mmas = 0;  // MMAs of a tile (one product)
+    size_t plane = 0, in_bytes = 0, smem = 0;
 };
 
-inline WideGeom tc_wide_geom(int R, int nr, bool split, int nbuf = 2)
+inline BlockTile tc_block_geom(int R, bool tf32, bool split, int gn, int nbuf)
 {
-    WideGeom g;
-    g.nkb = (128 + 2 * R + 15) / 16;
-    g.strip_len = 2 * g.nkb + 15;
-    g.delta = std::max(2 * g.nkb, (127 + 2 * R) / 8 + 1);
-    g.hs = (nr + 2 * R) | 1;  // odd chunk-column height: conflict-free staging stores
+    BlockTile g;
+    const int ce = tf32 ? 4 : 8, rows = 16 * gn + 2 * R;
+    g.gn = gn;
     g.nbuf = nbuf;
-    g.strip_bytes = (size_t)(2 * R * g.delta + g.strip_len) * 128;
-    g.in_bytes = (size_t)(2 * g.nkb) * g.hs * 16;
-    // 1 KB header, weight strips (hi, lo), nbuf input buffers (hi, lo)
-    g.smem = 1024 + (g.strip_bytes + nbuf * g.in_bytes) * (split ? 2 : 1);
+    g.nc = (8 + 2 * R + ce - 1) / ce;
+    g.pc = tf32 ? 8 + (g.nc - 1) / 2 : 7 + g.nc;
+    g.mmas = (16 + 2 * R) / 2 * g.nc;
+    const size_t row = (size_t)g.pc * 16;
+    // TF32: the odd-chunk plane starts 64 bytes off a 128-byte boundary
+    // distance, so that a quarter warp's four even and four odd chunks hit
+    // distinct banks
+    g.plane = tf32 ? ((size_t)rows * row + 127) / 128 * 128 + 64 : 0;
+    g.in_bytes = ((tf32 ? g.plane : 0) + (size_t)rows * row + 127) / 128 * 128;
+    // 1 KB header, 8 epilogue warps' staging (4 x 72 FP32), strips, buffers
+    g.smem = 1024 + 8 * 4 * 72 * 4 +
+             ((size_t)(31 + 2 * R) * g.nc * 128 + nbuf * g.in_bytes) * (split ? 2 : 1);
     return g;
 }
 
-// Tile of the wide kernel: output rows (MMA N) and input buffers -- the
-// first of (256, 2), (128, 2), (128, 1) whose operands fit in 227 KB (double
-// buffering overlaps the next tile's conversion with this tile's MMAs; one
-// buffer keeps N = 128 for the hi + lo forms at R = 7 .. 12).  Every R <= 12
-// fits; nr = 0 beyond.
-struct WideTile {
-    int nr = 0, nbuf = 0;
-};
-
-inline WideTile tc_wide_tile(int r, int t, bool split)
+// The tile of a grid with ny interior rows and ex stored columns on `sms` SMs:
+// the least (rounds of CTAs) x (cycles per tile) over gn = 32 .. 4 and two
+// operand buffers or one (one only where no two fit at that gn).  Cycles per
+// tile: the MMAs (90 cycles each until N / 2 is longer; see plan.cpp) and the
+// staging of its rows (1.2 cycles per 16 bytes), overlapped with two buffers
+// and in turn with one, plus a fixed 1500.
+inline BlockTile tc_block_tile(int R, bool tf32, bool split, int64_t ny, int64_t ex, int sms)
 {
-    WideTile w;
-    if (t * r > 12) return w;
-    const int cand[3][2] = {{256, 2}, {128, 2}, {128, 1}};
-    for (auto &c : cand)
-        if (tc_wide_geom(t * r, c[0], split, c[1]).smem <= 227 * 1024) {
-            w.nr = c[0];
-            w.nbuf = c[1];
-            return w;
+    BlockTile best;
+    double best_cost = 0;
+    for (int gn : {32, 24, 16, 12, 8, 6, 4}) {
+        // N = 8 gn: a multiple of 16 up to 256; TF32x3 keeps two accumulators per tile in TMEM
+        if (8 * gn * (tf32 && split ? 4 : 2) > 512) continue;
+        for (int nbuf : {2, 1}) {
+            const BlockTile g = tc_block_geom(R, tf32, split, gn, nbuf);
+            if (g.smem > 227 * 1024) continue;
+            const double mma = g.mmas * (split ? 3.0 : 1.0) * std::max(90.0, 4.0 * gn);
+            const double load = 1.2 * (16 * gn + 2 * R) * 2 * g.pc;
+            const int64_t tiles = ((ny + 16 * gn - 1) / (16 * gn)) * ((ex + 3 + 63) / 64);
+            const double cost =
+                (double)((tiles + sms - 1) / sms) * ((nbuf == 2 ? std::max(mma, load) : mma + load) + 1500.0);
+            if (best.gn == 0 || cost < 0.999 * best_cost) {
+                best = g;
+                best_cost = cost;
+            }
+            break;
         }
-    return w;
+    }
+    return best;
 }
-
-// Output rows per tile (MMA N) of the wide kernel, 0 if no tile fits.
-inline int tc_wide_nrows(int r, int t, bool split) { return tc_wide_tile(r, t, split).nr; }
 
 // 3-D wide FP16 kernel (tc3d_wide, one step per sweep): the Toeplitz factor
 // of line (dz, dy) is the A operand as in tc2d_wide (one strip per line, two
