@@ -41,17 +41,29 @@
 // at 2^-14, so values down to 2^-21 of the tile's largest keep 11 bits, and the
 // lo parts of f16x3 stay exact to 2^-31 of it).  TF32 needs no scale.
 //
-// Persistent, warp specialised, one CTA per SM (672 threads): warps 0-11 load
-// and convert the next tile into the other operand buffer, one thread of warp
-// 20 issues the MMAs into the other TMEM accumulator, warps 12-19 read the
-// previous accumulator back (tcgen05.ld), turn each 4 x 64 group of outputs
-// through shared memory and store whole rows.  Every wait is bounded.  Only
+// A tile is hx = 1 or 2 such column groups of 64 side by side: an MMA of N = 128
+// takes exactly half the time of one of N = 256 (64 / 128 cycles; ~50 is the
+// least), so the f16 form takes 256 x 128 tiles (N = 128 twice), whose rows
+// load in longer runs with less halo than 512 x 64.
+//
+// Persistent, warp specialised, one CTA per SM (768 threads): warps 0-14 load
+// and convert the next tile into the other operand buffer (each thread keeps
+// kBatch 16-byte loads in flight and starts the next tile's before the scale
+// exchange), warp 23 issues the MMAs into the other TMEM accumulator, warps
+// 15-22 read the previous accumulator back (tcgen05.ld), turn each 4 x 64 group
+// of outputs through shared memory and store whole rows.  The MMA warp runs its
+// loop converged with one elected lane issuing and the chunk count a
+// compile-time constant: issued by a single diverged lane with run-time
+// addressing, an MMA took ~70 cycles longer than its arithmetic (196 instead of
+// 128 at N = 256, 133 instead of 64 at N = 128).  Every wait is bounded.  Only
 // interior points farther than (t-1) r from the boundary are written; the
 // CUDA-core band kernel computes the others.
 //
-// Measured against the line form this replaced (Box-2D2R, one fused sweep):
-// f16 t = 4 on 16384^2 776 -> 572 us (HBM floor 317), f16x3 t = 4 on
-// 7001 x 6007 (unaligned rows) 433 -> 214 us.
+// Measured, one fused sweep (line form before, block form now): Box-2D2R f16
+// t = 4 on 16384^2 776 -> 476 us (HBM floor 317; a plain tiled copy that
+// re-reads the same halo 415), f16x3 t = 4 on 7001 x 6007 (unaligned rows)
+// 433 -> 171 us, Box-2D1R TF32 t = 7 on 10240^2 654 (2:4 sparse form) -> 265 us.
+// The loaders set the pace (15k cycles per 256 x 128 tile; MMAs 6.2k).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -59,6 +71,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "launch.h"
@@ -82,15 +95,14 @@ __host__ __device__ constexpr bool is_tf32(int f) { return f == kTF32 || f == kT
 constexpr int kMaxR = kWideMaxR;
 constexpr int kMaxLines = 2 * kMaxR + 1;
 constexpr int kBY = 16;                       // rows of an output block (16 x 8: MMA M = 128)
-constexpr int kTX = 64;                       // output columns per tile: 8 blocks
-constexpr int kLoadWarps = 12;                // warps 0-11
+constexpr int kTX = 64;                       // output columns of one MMA: 8 blocks
+constexpr int kLoadWarps = 15;                // warps 0-14
 constexpr int kLoaders = 32 * kLoadWarps;
-constexpr int kEpiWarp = kLoadWarps;          // warps 12-19: TMEM lane quarter w % 4, half (w - 12) / 4
+constexpr int kEpiWarp = kLoadWarps;          // warps 15-22: TMEM lane quarter w % 4, two warps each
 constexpr int kEpiWarps = 8;
-constexpr int kMmaWarp = kLoadWarps + kEpiWarps;  // warp 20
+constexpr int kMmaWarp = kLoadWarps + kEpiWarps;  // warp 23
 constexpr int kThreads = 32 * (kMmaWarp + 1);
-constexpr int kBatch = 8;                     // independent 16-byte loads in flight per loader thread
-constexpr int kBatchU = 4;                    // the same where a quad takes two (unaligned rows)
+constexpr int kBatch = 8;                     // 16-byte loads kept in flight per loader thread
 constexpr int kHeader = 1024;
 constexpr int kStageRow = kTX + 8;             // epilogue staging: 4 rows of 64 outputs per warp, padded
 constexpr int kStageBytes = kEpiWarps * 4 * kStageRow * 4;
@@ -101,6 +113,7 @@ struct WideParams {
     double w[kMaxLines * kMaxLines];  // composite w^(t), (2R+1) x (2R+1), row-major
     int R, rh, band, ew;
     int gn;     // block rows per tile: 16 gn output rows, MMA N = 8 gn
+    int hx;     // 64-column halves per tile, each with MMAs of its own
     int nbuf;   // operand buffers (2, or 1 where two do not fit)
     int nc;     // 16-byte chunks of a neighbourhood row (8 + 2R columns)
     int pc;     // 8-column units of a staged row
@@ -209,7 +222,7 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
     uint64_t *eub = reinterpret_cast<uint64_t *>(smem + 80);      // [4] a tile's scale published
     int *wmax = reinterpret_cast<int *>(smem + 128);              // [2][kLoadWarps]
     int *eus = reinterpret_cast<int *>(smem + 256);               // [4] input scale exponent per tile
-    const int R = p.R, lines = 2 * R + 1, nc = p.nc, pc = p.pc, gn = p.gn, nbuf = p.nbuf;
+    const int R = p.R, lines = 2 * R + 1, nc = p.nc, pc = p.pc, gn = p.gn, hx = p.hx, nbuf = p.nbuf;
     const uint32_t strip_bytes = (uint32_t)(31 + 2 * R) * nc * 128;
     const uint32_t in_bytes = p.in_bytes;
     float *stage = reinterpret_cast<float *>(smem + kHeader);
@@ -222,7 +235,7 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
     const int64_t Ey = p.Ey, Ex = p.Ex, rh = p.rh;
     const int64_t ny = Ey - 2 * rh;
     const int N = 8 * gn;                                  // MMA columns
-    const uint32_t aset = (uint32_t)N * (CORR ? 2 : 1);    // TMEM columns of one accumulator set
+    const uint32_t aset = (uint32_t)(N * hx) * (CORR ? 2 : 1);  // TMEM columns of one accumulator set
 
     if (warp == kMmaWarp) tmem_alloc(tmem_slot, 512);
     if (tid == 0) {
@@ -275,54 +288,76 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
     };
     auto origin = [&](int id, int64_t *Y0, int64_t *X0) {
         *Y0 = rh + (int64_t)(id / ntx) * (kBY * gn);
-        *X0 = (int64_t)(id % ntx) * kTX - p.xshift;
+        *X0 = (int64_t)(id % ntx) * (kTX * hx) - p.xshift;
     };
 
     if (warp == kMmaWarp) {
-        // ---------------- MMA issuer ----------------
-        if (lane == 0) {
+        // ---------------- MMA issuer (the whole warp; one elected lane issues) ----------------
+        auto mma_loop = [&](auto nc_const, auto hx_const) {
+            constexpr int NC = decltype(nc_const)::value, HX = decltype(hx_const)::value;
+            const uint32_t leader = elect_lane();
             const uint32_t idesc = instr_desc(TF ? kFmtTF32 : (FORM == kBF16x3 ? kFmtBF16 : kFmtF16), 128, N);
             const uint32_t wbase = smem_u32(Whi), rowb = (uint32_t)pc * 16;
-            const uint64_t a_c = smem_desc(wbase, 128, (uint32_t)nc * 128);       // chunk pairs of one row
-            const uint64_t a_r = smem_desc(wbase, (uint32_t)nc * 128, (uint32_t)nc * 128);  // one chunk of two rows
-            const uint64_t dlo_a = (uint64_t)(strip_bytes >> 4), dlo_b = (uint64_t)((nbuf * in_bytes) >> 4);
+            // descriptors of chunk pairs of one row (c) and of one chunk of two rows (r): the low
+            // word holds LBO and the start address, which advances; SBO sits in the high word
+            const uint64_t a_c = smem_desc(wbase, 128, NC * 128), a_r = smem_desc(wbase, NC * 128, NC * 128);
+            const uint32_t ahi = (uint32_t)(a_c >> 32), ac0 = (uint32_t)a_c, ar0 = (uint32_t)a_r;
+            const uint32_t dlo_a = strip_bytes >> 4, dlo_b = (nbuf * in_bytes) >> 4;
+            const uint32_t n_tmem = (uint32_t)N;
             int k = 0;
             for (int id = blockIdx.x; id < ntiles; id += gridDim.x, ++k) {
                 const int b = k & 1;
-                if (!bounded_wait(&full[b], (k >> 1) & 1, kWaitCycles)) break;
-                if (k >= 2 && !bounded_wait(&accfree[b], ((k - 2) >> 1) & 1, kWaitCycles)) break;
+                bool up = bounded_wait(&full[b], (k >> 1) & 1, kWaitCycles);
+                if (k >= 2) up = up && bounded_wait(&accfree[b], ((k - 2) >> 1) & 1, kWaitCycles);
+                if (!__all_sync(0xffffffffu, up)) break;
                 fence_after_thread_sync();
                 const uint32_t ib = smem_u32(ibase + (nbuf == 2 ? b : 0) * in_bytes);
-                const uint64_t b_c = smem_desc(ib, TF ? p.plane : 16u, 16 * rowb);
-                const uint64_t b_r = smem_desc(ib, rowb, 16 * rowb);
-                const uint32_t d = tmem + (uint32_t)b * aset, dc = d + (uint32_t)N;
-                uint32_t acc = 0;
-                auto issue = [&](uint64_t da, uint64_t db) {
-                    if constexpr (TF) {
-                        mma_tf32(d, da, db, idesc, acc);
-                        if (SPLIT) {
-                            mma_tf32(dc, da, db + dlo_b, idesc, acc);
-                            mma_tf32(dc, da + dlo_a, db, idesc, 1);
-                        }
-                    } else {
-                        mma_f16(d, da, db, idesc, acc);
-                        if (SPLIT) {
-                            mma_f16(d, da, db + dlo_b, idesc, 1);
-                            mma_f16(d, da + dlo_a, db, idesc, 1);
+                const uint64_t b_c = smem_desc(ib, TF ? p.plane : 16u, 16 * rowb), b_r = smem_desc(ib, rowb, 16 * rowb);
+                const uint32_t bhi = (uint32_t)(b_c >> 32);
+                uint32_t ac = ac0, ar = ar0, bc = (uint32_t)b_c, br = (uint32_t)b_r;
+                const uint32_t d0 = tmem + (uint32_t)b * aset;
+                // one K step of every column group; FIRST: the accumulators start at zero
+                auto issue = [&](auto first, uint32_t da, uint32_t db) {
+                    constexpr int ACC = decltype(first)::value ? 0 : 1;
+#pragma unroll
+                    for (int h = 0; h < HX; ++h) {
+                        const uint32_t d = d0 + h * n_tmem, dbh = db + 8 * h;  // 8 units: the next 64 columns
+                        if constexpr (TF) {
+                            mma_tf32_warp<ACC>(leader, d, da, ahi, dbh, bhi, idesc);
+                            if constexpr (SPLIT) {
+                                const uint32_t dc = d + HX * n_tmem;
+                                mma_tf32_warp<ACC>(leader, dc, da, ahi, dbh + dlo_b, bhi, idesc);
+                                mma_tf32_warp<1>(leader, dc, da + dlo_a, ahi, dbh, bhi, idesc);
+                            }
+                        } else {
+                            mma_f16_warp<ACC>(leader, d, da, ahi, dbh, bhi, idesc);
+                            if constexpr (SPLIT) {
+                                mma_f16_warp<1>(leader, d, da, ahi, dbh + dlo_b, bhi, idesc);
+                                mma_f16_warp<1>(leader, d, da + dlo_a, ahi, dbh, bhi, idesc);
+                            }
                         }
                     }
-                    acc = 1;
                 };
-                for (int ky = 0; ky < kBY + 2 * R; ky += 2) {
-                    for (int y = ky; y < ky + 2; ++y)
-                        for (int c = 0; c + 1 < nc; c += 2)
-                            issue(a_c + (uint64_t)(y * nc + c) * 8, b_c + (uint64_t)(y * pc + (TF ? c / 2 : c)));
-                    if (nc & 1) {
-                        const int c = nc - 1;
-                        issue(a_r + (uint64_t)(ky * nc + c) * 8, b_r + (uint64_t)(ky * pc + (TF ? c / 2 : c)));
-                    }
-                }
-                mma_commit(&done[b]);
+                auto two_rows = [&](auto first) {
+                    constexpr bool F = decltype(first)::value;
+#pragma unroll
+                    for (int y = 0; y < 2; ++y)
+#pragma unroll
+                        for (int c = 0; c + 1 < NC; c += 2) {
+                            const uint32_t da = ac + (y * NC + c) * 8, db = bc + (y ? pc : 0) + (TF ? c / 2 : c);
+                            if (F && y == 0 && c == 0) issue(std::true_type{}, da, db);
+                            else issue(std::false_type{}, da, db);
+                        }
+                    if constexpr ((NC & 1) != 0)
+                        issue(std::false_type{}, ar + (NC - 1) * 8, br + (TF ? (NC - 1) / 2 : NC - 1));
+                    ac += 2 * NC * 8;
+                    ar += 2 * NC * 8;
+                    bc += (uint32_t)(2 * pc);
+                    br += (uint32_t)(2 * pc);
+                };
+                two_rows(std::true_type{});
+                for (int ky = 2; ky < kBY + 2 * R; ky += 2) two_rows(std::false_type{});
+                mma_commit_warp(leader, &done[b]);
             }
             // the last tiles' MMAs complete before the TMEM is released
             for (int j = k - 2; j < k; ++j)
@@ -331,6 +366,19 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
                     while (!mbar_try_wait(&done[j & 1], (j >> 1) & 1) && clock64() - t0 < kWaitCycles) {
                     }
                 }
+        };
+        auto with_hx = [&](auto nc_const) {
+            if (hx == 2) mma_loop(nc_const, std::integral_constant<int, 2>{});
+            else mma_loop(nc_const, std::integral_constant<int, 1>{});
+        };
+        switch (nc) {
+        case 2: if constexpr (!TF) with_hx(std::integral_constant<int, 2>{}); break;
+        case 3: with_hx(std::integral_constant<int, 3>{}); break;
+        case 4: with_hx(std::integral_constant<int, 4>{}); break;
+        case 5: if constexpr (TF) with_hx(std::integral_constant<int, 5>{}); break;
+        case 6: if constexpr (TF) with_hx(std::integral_constant<int, 6>{}); break;
+        case 7: if constexpr (TF) with_hx(std::integral_constant<int, 7>{}); break;
+        case 8: if constexpr (TF) with_hx(std::integral_constant<int, 8>{}); break;
         }
         __syncwarp();
     } else if (warp < kEpiWarp) {
@@ -341,117 +389,128 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
         // thread tid takes the items i = tid + m kLoaders; (row, quad) advance by a constant step
         const int row0 = tid / F4, col0 = tid - row0 * F4;
         const int step_r = kLoaders / F4, step_c = kLoaders - step_r * F4;
-        // ask L2 for tile `id`'s input rows (one prefetch per 128 bytes, every
-        // address inside the stored array), so that its loads wait on L2 rather
-        // than DRAM latency
-        auto prefetch_l2 = [&](int id) {
-            int64_t Y0, X0;
-            origin(id, &Y0, &X0);
-            const int64_t gx_lo = max((int64_t)0, X0 - R), gx_hi = min(Ex, X0 - R + 8 * pc);
-            if (gx_lo >= gx_hi) return;
-            const int segs = (int)((gx_hi - gx_lo + 31) / 32);
-            for (int e = tid; e < rows * segs; e += kLoaders) {
-                const int row = e / segs, l = e - (e / segs) * segs;
-                const int64_t gy = Y0 - R + row;
-                if (gy < 0 || gy >= Ey) continue;
-                const int64_t gx = min(gx_lo + 32 * (int64_t)l, gx_hi - 1);
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(in + gy * Ex + gx));
+        const int64_t wrap = Ex - 4 * F4, step = step_r * Ex + 4 * step_c;
+        const float *q = in;  // the next item to load: its address
+        int c4 = 0;           // and its quad of the row
+        auto next = [&] {
+            q += step;
+            c4 += step_c;
+            if (c4 >= F4) {
+                c4 -= F4;
+                q += wrap;
             }
         };
+        // the staged region lies inside the stored array (no bounds tests), and
+        // its rows are 16-byte aligned
+        auto is_fast = [&](int64_t Y0, int64_t X0) {
+            return vec16 && X0 - R >= 0 && X0 - R + 8 * pc <= Ex && Y0 - R >= 0 && Y0 - R + rows <= Ey;
+        };
+        float4 v[kBatch] = {};  // loads in flight: items of the current (fast) tile
+        auto start_tile = [&](int64_t Y0, int64_t X0) {
+            q = in + (Y0 - R + row0) * Ex + (X0 - R + 4 * col0);
+            c4 = col0;
+        };
+        auto start_fast = [&](int64_t Y0, int64_t X0) {
+            start_tile(Y0, X0);
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (tid + u * kLoaders < items) v[u] = __ldcg(reinterpret_cast<const float4 *>(q));
+                next();
+            }
+        };
+        bool started = false;  // v holds this tile's first items
         int es = 12;  // the scale the next tile is first tried with: the previous tile's
         int k = 0;
         for (int id = blockIdx.x; id < ntiles; id += gridDim.x, ++k) {
             const int b = k & 1;
             int64_t Y0, X0;
             origin(id, &Y0, &X0);
-            if (id + (int)gridDim.x < ntiles) prefetch_l2(id + gridDim.x);
             // the operand buffer is free once the MMAs of tile k - nbuf completed
             if (nbuf == 2 && k >= 2 && !bounded_wait(&done[b], ((k - 2) >> 1) & 1, kWaitCycles)) break;
             if (nbuf == 1 && k >= 1 && !bounded_wait(&done[b ^ 1], ((k - 1) >> 1) & 1, kWaitCycles)) break;
             unsigned char *hi = ibase + (nbuf == 2 ? b : 0) * in_bytes, *lo = hi + nbuf * in_bytes;
-            // Interior tiles (the staged region inside the stored array): no
-            // per-load bounds tests.  Rows that are not 16-byte multiples are
-            // read as the two aligned 16-byte words around each quad (the
-            // region then keeps a stored row free above and below, so both
-            // words lie inside the array).
-            const bool inx = X0 - R >= 0 && X0 - R + 8 * pc <= Ex;
-            const bool fast = vec16 && inx && Y0 - R >= 0 && Y0 - R + rows <= Ey;
-            const bool fast_u = !vec16 && inx && Y0 - R >= 1 && Y0 - R + rows + 1 <= Ey;
-            const int64_t wrap = Ex - 4 * F4, step = step_r * Ex + 4 * step_c;
+            // Interior tiles: no per-load bounds tests.  Rows that are not 16-byte
+            // multiples are read as the two aligned 16-byte words around each
+            // quad (the region then keeps a stored row free above and below, so
+            // both words lie inside the array).
+            const bool fast = is_fast(Y0, X0);
+            const bool fast_u = !vec16 && X0 - R >= 0 && X0 - R + 8 * pc <= Ex && Y0 - R >= 1 &&
+                                Y0 - R + rows + 1 <= Ey;
             for (int attempt = 0;; ++attempt) {
                 const float xs = SCALED ? pow2f(es) : 1.0f;
                 unsigned mxu = 0;
-                auto use = [&](int i, const float4 &v) {
-                    if (SCALED) mxu = max_abs(mxu, v);
-                    put<FORM>(hi, lo, i, v, xs, p.plane);
-                };
-                const float *q = in + (Y0 - R + row0) * Ex + (X0 - R + 4 * col0);
-                int c4 = col0;
-                auto next = [&] {
-                    q += step;
-                    c4 += step_c;
-                    if (c4 >= F4) {
-                        c4 -= F4;
-                        q += wrap;
-                    }
+                auto use = [&](int i, const float4 &x) {
+                    if (SCALED) mxu = max_abs(mxu, x);
+                    put<FORM>(hi, lo, i, x, xs, p.plane);
                 };
                 if (fast) {
+                    if (!started) start_fast(Y0, X0);
                     for (int i0 = tid; i0 < items; i0 += kBatch * kLoaders) {
-                        float4 v[kBatch];
 #pragma unroll
                         for (int u = 0; u < kBatch; ++u) {
-                            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (i0 + u * kLoaders < items) v[u] = __ldcg(reinterpret_cast<const float4 *>(q));
+                            const int i = i0 + u * kLoaders;
+                            if (i < items) use(i, v[u]);
+                            if (i + kBatch * kLoaders < items) v[u] = __ldcg(reinterpret_cast<const float4 *>(q));
                             next();
                         }
-#pragma unroll
-                        for (int u = 0; u < kBatch; ++u)
-                            if (i0 + u * kLoaders < items) use(i0 + u * kLoaders, v[u]);
+                    }
+                    started = false;
+                    // the next tile's first loads run during the exchange and the waits
+                    if (attempt == 0 && id + (int)gridDim.x < ntiles) {
+                        int64_t Y1, X1;
+                        origin(id + gridDim.x, &Y1, &X1);
+                        if (is_fast(Y1, X1)) {
+                            start_fast(Y1, X1);
+                            started = true;
+                        }
                     }
                 } else if (fast_u) {
-                    for (int i0 = tid; i0 < items; i0 += kBatchU * kLoaders) {
-                        float4 a[kBatchU], e[kBatchU];
+                    start_tile(Y0, X0);
+                    constexpr int U = kBatch / 2;  // v[u], v[U + u]: the two words of a quad
+                    for (int i0 = tid; i0 < items; i0 += U * kLoaders) {
                         int sh = 0;
 #pragma unroll
-                        for (int u = 0; u < kBatchU; ++u) {
-                            a[u] = e[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        for (int u = 0; u < U; ++u) {
                             const int s = (int)(reinterpret_cast<uintptr_t>(q) >> 2) & 3;
                             sh |= s << (2 * u);
                             if (i0 + u * kLoaders < items) {
                                 const float4 *a4 = reinterpret_cast<const float4 *>(q - s);
-                                a[u] = __ldg(a4);
-                                if (s) e[u] = __ldg(a4 + 1);
+                                v[u] = __ldg(a4);
+                                if (s) v[U + u] = __ldg(a4 + 1);
                             }
                             next();
                         }
 #pragma unroll
-                        for (int u = 0; u < kBatchU; ++u) {
+                        for (int u = 0; u < U; ++u) {
                             if (i0 + u * kLoaders >= items) continue;
                             // quad = values s .. s + 3 of (a, e): shift by two, then by one
                             const int s = sh >> (2 * u);
-                            const float4 a2 = (s & 2) ? make_float4(a[u].z, a[u].w, e[u].x, e[u].y) : a[u];
-                            const float n4 = (s & 2) ? e[u].z : e[u].x;
+                            const float4 a = v[u], e = v[U + u];
+                            const float4 a2 = (s & 2) ? make_float4(a.z, a.w, e.x, e.y) : a;
+                            const float n4 = (s & 2) ? e.z : e.x;
                             use(i0 + u * kLoaders, (s & 1) ? make_float4(a2.y, a2.z, a2.w, n4) : a2);
                         }
                     }
                 } else {
                     // edge tiles: every value tested; cells outside the stored array are zero
+                    start_tile(Y0, X0);
                     int row = row0;
                     for (int i = tid; i < items; i += kLoaders) {
                         const int64_t gy = Y0 - R + row, gx = X0 - R + 4 * c4;
-                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (gy >= 0 && gy < Ey) {
                             if (vec16) {
                                 // X0 - R is a multiple of 4: the quad lies wholly inside or outside the row
-                                if (gx >= 0 && gx < Ex) v = __ldcg(reinterpret_cast<const float4 *>(q));
+                                if (gx >= 0 && gx < Ex) x = __ldcg(reinterpret_cast<const float4 *>(q));
                             } else {
-                                if (gx >= 0 && gx < Ex) v.x = __ldcg(q);
-                                if (gx + 1 >= 0 && gx + 1 < Ex) v.y = __ldcg(q + 1);
-                                if (gx + 2 >= 0 && gx + 2 < Ex) v.z = __ldcg(q + 2);
-                                if (gx + 3 >= 0 && gx + 3 < Ex) v.w = __ldcg(q + 3);
+                                if (gx >= 0 && gx < Ex) x.x = __ldcg(q);
+                                if (gx + 1 >= 0 && gx + 1 < Ex) x.y = __ldcg(q + 1);
+                                if (gx + 2 >= 0 && gx + 2 < Ex) x.z = __ldcg(q + 2);
+                                if (gx + 3 >= 0 && gx + 3 < Ex) x.w = __ldcg(q + 3);
                             }
                         }
-                        use(i, v);
+                        use(i, x);
                         row += step_r + (c4 + step_c >= F4);
                         next();
                     }
@@ -472,6 +531,7 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
                 const int top = emax - 126 + es;
                 if (emax == 0 || (top <= 15 && top >= 8)) break;
                 es = max(-126, min(127, 138 - emax));
+                started = false;  // converting again reloads the tile into v
             }
             if (*(volatile int *)abort_flag) break;
             // publish the scale: slot k & 3 was last read by the epilogue of tile
@@ -485,11 +545,11 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
             mbar_arrive(&full[b]);
         }
     } else {
-        // ---------------- epilogue (warps 12-19) ----------------
+        // ---------------- epilogue (warps 15-22) ----------------
         // warp w reads TMEM lanes 32 q .. 32 q + 31 (q = w % 4, the lane quarter
-        // a warp may access): rows 12 - 4q .. 15 - 4q of every block; half h of
-        // the block-row pairs
-        const int q = (warp - kEpiWarp) & 3, h = (warp - kEpiWarp) >> 2;
+        // a warp may access): rows 12 - 4q .. 15 - 4q of every block; every
+        // other pair of block rows
+        const int q = warp & 3, h = (warp - kEpiWarp) >> 2;
         const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16);
         float *st = stage + (warp - kEpiWarp) * 4 * kStageRow;
         float *put_at = st + (3 - (lane >> 3)) * kStageRow + 7 - (lane & 7);
@@ -512,21 +572,26 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
             fence_after_thread_sync();
             int64_t Y0, X0;
             origin(id, &Y0, &X0);
-            // written columns [x_lo, x_hi) and rows [y_lo, y_hi) of the tile
-            const int x_lo = (int)max((int64_t)0, rh + p.band - X0), x_hi = (int)min((int64_t)kTX, Ex - rh - p.band - X0);
+            // written rows [y_lo, y_hi) of the tile
             const int y_lo = (int)max((int64_t)0, p.band - (Y0 - rh));
             const int y_hi = (int)min((int64_t)kBY * gn, ny - p.band - (Y0 - rh));
-            const int vst = x_lo == 0 && x_hi == kTX ? p.vst : 0;
             // out = acc 2^(ew - 15 - es), as two in-range powers of two
             const int e = p.ew - 15 - es, e1 = e / 2, e2 = e - e1;
             const float s1 = SCALED ? pow2f(max(-126, min(127, e1))) : 1.0f;
             const float s2 = SCALED ? pow2f(max(-126, min(127, e2))) : 1.0f;
-            float *const o = out + Y0 * Ex + X0;
-            for (int g2 = 2 * h; g2 < gn; g2 += 4) {
+            for (int pr = h; pr < hx * (gn / 2); pr += 2) {
+                const int hc = pr >= gn / 2, g2 = 2 * (pr - hc * (gn / 2));  // column half, first block row
+                // written columns [x_lo, x_hi) of the half
+                const int64_t gx0 = X0 + hc * kTX;
+                const int x_lo = (int)max((int64_t)0, rh + p.band - gx0);
+                const int x_hi = (int)min((int64_t)kTX, Ex - rh - p.band - gx0);
+                const int vst = x_lo == 0 && x_hi == kTX ? p.vst : 0;
+                float *const o = out + Y0 * Ex + gx0;
+                const uint32_t col = (uint32_t)b * aset + (uint32_t)(hc * N + 8 * g2);
                 uint32_t v[16], c[16];
                 __syncwarp();
-                tmem_ld_32x32b_x16(lane_base + (uint32_t)b * aset + (uint32_t)(8 * g2), v);
-                if (CORR) tmem_ld_32x32b_x16(lane_base + (uint32_t)b * aset + (uint32_t)(N + 8 * g2), c);
+                tmem_ld_32x32b_x16(lane_base + col, v);
+                if (CORR) tmem_ld_32x32b_x16(lane_base + col + (uint32_t)(N * hx), c);
                 tmem_ld_wait();
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
@@ -627,6 +692,7 @@ stencil_status launch_form(const Plan &p, const void *in, void *out, int t, cuda
     wp.rh = r;
     wp.band = (t - 1) * r;
     wp.gn = g.gn;
+    wp.hx = g.hx;
     wp.nbuf = g.nbuf;
     wp.nc = g.nc;
     wp.pc = g.pc;
@@ -650,7 +716,7 @@ stencil_status launch_form(const Plan &p, const void *in, void *out, int t, cuda
     }();
     stencil_status s = ensure_smem((const void *)kern, g.smem);
     if (s != STENCIL_OK) return s;
-    const int64_t nty = (p.dims[1] + kBY * g.gn - 1) / (kBY * g.gn), ntx = (p.ext[2] + wp.xshift + kTX - 1) / kTX;
+    const int64_t nty = (p.dims[1] + kBY * g.gn - 1) / (kBY * g.gn), ntx = (p.ext[2] + wp.xshift + kTX * g.hx - 1) / (kTX * g.hx);
     const int64_t ntiles = nty * ntx;
     if (ntiles > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const unsigned grid = (unsigned)std::min<int64_t>(ntiles, sms);

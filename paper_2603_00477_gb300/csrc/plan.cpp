@@ -497,13 +497,13 @@ static stencil_status enumerate(Plan *p, std::vector<Cand> *out)
                         c.tile[1] = tc_wide3_nrows(shape, r);  // one plane: rows (MMA N) x 128 columns
                         c.tile[2] = 128;
                     } else if (p->dtype == STENCIL_F32 && path == STENCIL_PATH_TENSOR_CORE) {
-                        // the block kernels (k_wide.cu): 16 gn output rows x 64 columns
+                        // the block kernels (k_wide.cu): 16 gn output rows x 64 hx columns
                         const bool tf = prec == STENCIL_PREC_TF32 || prec == STENCIL_PREC_TF32X3;
                         const BlockTile bt = tc_block_tile(
                             t * r, tf, prec != STENCIL_PREC_TF32 && prec != STENCIL_PREC_F16, p->dims[1], p->ext[2],
                             device_sms());
                         c.tile[1] = 16 * bt.gn;
-                        c.tile[2] = 64;
+                        c.tile[2] = 64 * bt.hx;
                     }
                     TcGeometry g = tc_geometry(shape, d, r, t, p->dtype, prec, path);
                     ModelOut m = model_eval(shape, d, r, t, D, g.sparsity, beta_of(prec, slices), P_cu,
@@ -545,6 +545,18 @@ stencil_status dispatch(Plan *p)
                                    x.prec == STENCIL_PREC_OZAKI ? 100.0 : beta_of(x.prec));
         };
         if (key(c) < key(*pick)) pick = &c;
+    }
+
+    // TF32 with the path left open: the ranking above sets t, the dense block
+    // kernel runs it.  The ranking's instruction roofs describe the line-form
+    // kernels, among which the sparse one led from t = 3; the block form
+    // (k_wide.cu) is faster than the sparse kernel at every t and radius
+    // measured.  The two forms round the same operands to TF32, so the choice
+    // changes results by FP32 accumulation order only, which a different t
+    // would not.
+    if (pick->path == STENCIL_PATH_SPARSE_TENSOR_CORE && p->req_path == STENCIL_PATH_AUTO) {
+        for (auto &c : cands)
+            if (c.path == STENCIL_PATH_TENSOR_CORE && c.prec == pick->prec && c.t == pick->t) pick = &c;
     }
 
     p->path = pick->path;

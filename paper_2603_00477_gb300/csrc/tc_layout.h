@@ -103,9 +103,11 @@ inline int tc_wide_nrows(int r, int t, bool split)
 
 // Block form of the 2-D kernels (k_wide.cu): MMA rows = the 16 x 8 outputs of a
 // block, MMA columns = 8 gn block positions (8 across, gn down), K = the
-// 16-byte chunks of the block's (16 + 2R) x (8 + 2R) neighbourhood.
+// 16-byte chunks of the block's (16 + 2R) x (8 + 2R) neighbourhood; a tile has
+// hx such groups of 64 columns side by side.
 struct BlockTile {
-    int gn = 0;    // block rows: the tile is 16 gn x 64 outputs (0: no tile)
+    int gn = 0;    // block rows: the tile is 16 gn x 64 hx outputs (0: no tile)
+    int hx = 1;
     int nbuf = 0;  // operand buffers
     int nc = 0;    // 16-byte chunks of a neighbourhood row
     int pc = 0;    // 8-column units of a staged row
@@ -113,15 +115,16 @@ struct BlockTile {
     size_t plane = 0, in_bytes = 0, smem = 0;
 };
 
-inline BlockTile tc_block_geom(int R, bool tf32, bool split, int gn, int nbuf)
+inline BlockTile tc_block_geom(int R, bool tf32, bool split, int gn, int hx, int nbuf)
 {
     BlockTile g;
     const int ce = tf32 ? 4 : 8, rows = 16 * gn + 2 * R;
     g.gn = gn;
+    g.hx = hx;
     g.nbuf = nbuf;
     g.nc = (8 + 2 * R + ce - 1) / ce;
-    g.pc = tf32 ? 8 + (g.nc - 1) / 2 : 7 + g.nc;
-    g.mmas = (16 + 2 * R) / 2 * g.nc;
+    g.pc = 8 * hx + (tf32 ? (g.nc - 1) / 2 : g.nc - 1);
+    g.mmas = (16 + 2 * R) / 2 * g.nc * hx;
     const size_t row = (size_t)g.pc * 16;
     // TF32: the odd-chunk plane starts 64 bytes off a 128-byte boundary
     // distance, so that a quarter warp's four even and four odd chunks hit
@@ -135,33 +138,37 @@ inline BlockTile tc_block_geom(int R, bool tf32, bool split, int gn, int nbuf)
 }
 
 // The tile of a grid with ny interior rows and ex stored columns on `sms` SMs:
-// the least (rounds of CTAs) x (cycles per tile) over gn = 32 .. 4 and two
-// operand buffers or one (one only where no two fit at that gn).  Cycles per
-// tile: the MMAs (90 cycles each until N / 2 is longer; see plan.cpp) and the
-// staging of its rows (1.2 cycles per 16 bytes), overlapped with two buffers
-// and in turn with one, plus a fixed 1500.
+// the least (rounds of CTAs) x (cycles per tile) over gn = 32 .. 4, hx = 2 or 1
+// and two operand buffers or one (one only where no two fit).  Cycles per
+// tile, measured: an MMA takes N / 2 = 4 gn cycles, at least 50; staging 1.0 per
+// 16 bytes; HBM 1.15 x 8 bytes per output at 21.5 bytes per cycle and SM.  They
+// overlap with two operand buffers; with one, staging and MMAs take turns.
+// 2000 cycles per tile do not overlap (first loads, scale exchange, hand-over).
 inline BlockTile tc_block_tile(int R, bool tf32, bool split, int64_t ny, int64_t ex, int sms)
 {
     BlockTile best;
     double best_cost = 0;
-    for (int gn : {32, 24, 16, 12, 8, 6, 4}) {
-        // N = 8 gn: a multiple of 16 up to 256; TF32x3 keeps two accumulators per tile in TMEM
-        if (8 * gn * (tf32 && split ? 4 : 2) > 512) continue;
-        for (int nbuf : {2, 1}) {
-            const BlockTile g = tc_block_geom(R, tf32, split, gn, nbuf);
-            if (g.smem > 227 * 1024) continue;
-            const double mma = g.mmas * (split ? 3.0 : 1.0) * std::max(90.0, 4.0 * gn);
-            const double load = 1.2 * (16 * gn + 2 * R) * 2 * g.pc;
-            const int64_t tiles = ((ny + 16 * gn - 1) / (16 * gn)) * ((ex + 3 + 63) / 64);
-            const double cost =
-                (double)((tiles + sms - 1) / sms) * ((nbuf == 2 ? std::max(mma, load) : mma + load) + 1500.0);
-            if (best.gn == 0 || cost < 0.999 * best_cost) {
-                best = g;
-                best_cost = cost;
+    for (int hx : {2, 1})
+        for (int gn : {32, 24, 16, 12, 8, 6, 4}) {
+            // N = 8 gn: a multiple of 16 up to 256; TMEM holds two sets of hx accumulators
+            // (TF32x3: two accumulators each)
+            if (8 * gn * hx * (tf32 && split ? 4 : 2) > 512) continue;
+            for (int nbuf : {2, 1}) {
+                const BlockTile g = tc_block_geom(R, tf32, split, gn, hx, nbuf);
+                if (g.smem > 227 * 1024) continue;
+                const double mma = g.mmas * (split ? 3.0 : 1.0) * std::max(50.0, 4.0 * gn);
+                const double load = 1.0 * (16 * gn + 2 * R) * 2 * g.pc;
+                const double hbm = 1.15 * 8.0 * (16.0 * gn * 64.0 * hx) / 21.5;
+                const int64_t tiles = ((ny + 16 * gn - 1) / (16 * gn)) * ((ex + 3 + 64 * hx - 1) / (64 * hx));
+                const double cost = (double)((tiles + sms - 1) / sms) *
+                                    (std::max(hbm, nbuf == 2 ? std::max(mma, load) : mma + load) + 2000.0);
+                if (best.gn == 0 || cost < 0.999 * best_cost) {
+                    best = g;
+                    best_cost = cost;
+                }
+                break;
             }
-            break;
         }
-    }
     return best;
 }
 

@@ -111,6 +111,59 @@ __device__ __forceinline__ void mma_commit(uint64_t *mbar)
                  : "memory");
 }
 
+// True in exactly one lane of a converged warp (always the same one).
+__device__ __forceinline__ uint32_t elect_lane()
+{
+    uint32_t v;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(v));
+    return v;
+}
+
+// The same MMAs executed by a whole converged warp, issued by its elected lane
+// (`leader`, from elect_lane): operands can stay in uniform registers.  The
+// descriptors come as low word (start address, the part that advances) and
+// high word; ACC is the accumulate flag.
+template <int ACC>
+__device__ __forceinline__ void mma_tf32_warp(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi,
+                                              uint32_t b_lo, uint32_t b_hi, uint32_t idesc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "setp.ne.b32 q, %7, 0;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %5, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC), "r"(leader)
+        : "memory");
+}
+
+template <int ACC>
+__device__ __forceinline__ void mma_f16_warp(uint32_t leader, uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi,
+                                             uint32_t b_lo, uint32_t b_hi, uint32_t idesc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "setp.ne.b32 q, %7, 0;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC), "r"(leader)
+        : "memory");
+}
+
+// mma_commit by the lane that issued the MMAs.
+__device__ __forceinline__ void mma_commit_warp(uint32_t leader, uint64_t *mbar)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(mbar)),
+        "r"(leader)
+        : "memory");
+}
+
 // ---- mbarrier --------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t *mbar, uint32_t count)
 {
