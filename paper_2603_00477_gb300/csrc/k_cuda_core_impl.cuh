@@ -17,6 +17,49 @@ template <typename T>
 constexpr int kV = sizeof(T) == 8 ? 4 : 8;  // strip height: FP64 needs fewer accumulators
 constexpr size_t kMaxSmem = 227 * 1024;
 
+// 2-D FP32, t = 1 or 2, radius <= 3: the marching kernel.  The segment of output
+// rows per work item is chosen so that the items fill k = 1 .. 4 rounds of the
+// resident warps: the time is ~ k (segment + 2 t r + a start-up of ~12 rows).
+template <int SHAPE, int R, int T, bool VEC>
+stencil_status launch2d_march(const Plan &p, const void *in, void *out, cudaStream_t st)
+{
+    using Wt = cu::Weights<float, cu::Taps<SHAPE, 2, R>::K>;
+    Wt wt;
+    for (int k = 0; k < cu::Taps<SHAPE, 2, R>::K; k++) wt.w[k] = (float)p.w[k];
+    auto kern = cu::cu2d_march<SHAPE, R, T, VEC>;
+    int occ = 0;
+    stencil_status s = occupancy((const void *)kern, cu::kMarchThreads, 0, &occ);
+    if (s != STENCIL_OK) return s;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    constexpr int CW = cu::march_cols<R, T>();
+    const int xb = R - R % 4;  // quads start on 16-byte boundaries of aligned rows
+    const int64_t ny = p.dims[1], ncb = (p.ext[2] - R - xb + CW - 1) / CW;
+    const int64_t warps = (int64_t)std::max(1, occ) * std::max(1, sms) * (cu::kMarchThreads / 32);
+    int64_t seg = 0, best = 0;
+    for (int64_t k = 1; k <= 4; k++) {
+        const int64_t nseg = std::min(ny, k * warps / ncb);
+        if (nseg < 1) continue;
+        const int64_t c = (ny + nseg - 1) / nseg, cost = k * (c + 2 * R * T + 12);
+        if (seg == 0 || cost < best) {
+            best = cost;
+            seg = c;
+        }
+    }
+    if (seg == 0) seg = ny;  // more column blocks than four rounds hold
+    const int64_t items = ncb * ((ny + seg - 1) / seg);
+    if (items > 0x7fffffff || seg > 0x3fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
+    const int64_t per_cta = cu::kMarchThreads / 32;
+    const unsigned grid =
+        (unsigned)std::min<int64_t>((items + per_cta - 1) / per_cta, (int64_t)std::max(1, occ) * std::max(1, sms));
+    kern<<<grid, cu::kMarchThreads, 0, st>>>((const float *)in, (float *)out, wt, p.ext[1], p.ext[2], (int)ncb,
+                                             (int)seg, (int)items, xb);
+    note_launch();
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu2d_march launch");
+}
+
 template <typename T, int SHAPE, int R>
 stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStream_t st)
 {
@@ -25,6 +68,22 @@ stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStr
     for (int k = 0; k < cu::Taps<SHAPE, 2, R>::K; k++) wt.w[k] = (T)p.w[k];
     int tile[3] = {p.tile[0], p.tile[1], p.tile[2]};
     if (p.path != STENCIL_PATH_CUDA_CORE) cu_default_tile(p, t, tile);
+    if constexpr (sizeof(T) == 4 && R <= (SHAPE == 0 ? 2 : 3)) {
+        // a tile asked for by option or picked by the autotuner runs the tiled kernel
+        int def[3];
+        cu_default_tile(p, p.t, def);
+        if (t <= 2 && tile[1] == def[1] && tile[2] == def[2]) {
+            const bool vec = p.ext[2] % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0 &&
+                             reinterpret_cast<uintptr_t>(out) % 16 == 0;
+            if (t == 1)
+                return vec ? launch2d_march<SHAPE, R, 1, true>(p, in, out, st)
+                           : launch2d_march<SHAPE, R, 1, false>(p, in, out, st);
+            // two steps where their partial sums and weights fit in registers
+            if constexpr (R == 1 || (SHAPE == 1 && R == 2))
+                return vec ? launch2d_march<SHAPE, R, 2, true>(p, in, out, st)
+                           : launch2d_march<SHAPE, R, 2, false>(p, in, out, st);
+        }
+    }
     const int BY = tile[1], BX = tile[2];
     const size_t H = BY + 2 * t * R, W = BX + 2 * t * R;
     const size_t bufb = cu::buf_elems<T>((int)H, (int)W) * sizeof(T);
