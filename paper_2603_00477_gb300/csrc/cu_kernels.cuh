@@ -1009,7 +1009,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 
 // ---------------------------------------------------------------------------
 // 3-D, one step per sweep (t = 1), 2.5-D streaming: a work item is a
-// (BY x BX) tile of one z chunk of CZ planes.  The CTA marches along z with a
+// (BY x BX) tile of one z chunk of cz planes.  The CTA marches along z with a
 // ring of NP = 2R + 1 + PF input planes (each the tile grown by R in y and x)
 // in shared memory: while plane z is computed, planes z + R + 1 ..
 // z + R + PF are in flight (cp.async, 16-byte copies where the stored rows
@@ -1019,8 +1019,6 @@ __global__ void __launch_bounds__(kThreads, 2)
 // y = ty + 16 i; each (oz, oy) row segment of 4 + 2R values is read with
 // 16-byte shared loads (rows padded to 16 bytes) and used for the 4 outputs.
 // ---------------------------------------------------------------------------
-constexpr int kStreamCZ = 64;
-
 template <typename T>
 __host__ __device__ constexpr int stream_rows_per_thread()
 {
@@ -1124,7 +1122,7 @@ template <typename T, int SHAPE, int R>
 __global__ void __launch_bounds__(kThreads, 2)
     cu3d_stream(const T *__restrict__ in, T *__restrict__ out,
                 const __grid_constant__ Weights<T, Taps<SHAPE, 3, R>::K> wt, int64_t Ez, int64_t Ey, int64_t Ex,
-                int tiles_x, int tiles_y, int chunks_z, int nitems)
+                int tiles_x, int tiles_y, int cz, int nitems)
 {
     constexpr int KT = Taps<SHAPE, 3, R>::K;
     constexpr bool kSmemW = sizeof(T) == 8;
@@ -1152,9 +1150,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
         const int bx = item % tiles_x, by = (item / tiles_x) % tiles_y, bz = item / (tiles_x * tiles_y);
         // stored coordinates of the first output of the item
-        const int64_t Z0 = R + (int64_t)bz * kStreamCZ, Y0 = R + (int64_t)by * BY, X0 = R + (int64_t)bx * BX;
+        const int64_t Z0 = R + (int64_t)bz * cz, Y0 = R + (int64_t)by * BY, X0 = R + (int64_t)bx * BX;
         const int64_t rem = nz - (Z0 - R);
-        const int nzo = (int)(rem < kStreamCZ ? rem : kStreamCZ);  // output planes of this item
+        const int nzo = (int)(rem < cz ? rem : cz);  // output planes of this item
         const int64_t zfirst = Z0 - R;                                // first input plane
         const int nin = nzo + 2 * R;                                  // input planes of the item
         // copy input plane gz (rows Y0-R.., columns X0-R.., zero outside the
