@@ -1244,40 +1244,42 @@ __global__ void __launch_bounds__(kThreads, 2)
 // ---------------------------------------------------------------------------
 // 3-D, t = 1, FP32: z-marching with rotating partial sums.
 // ---------------------------------------------------------------------------
-// A work item is a 64-column x BY-row tile and a run of cz output planes.
-// The CTA stages ONE input plane at a time (a ring of kRotNPL planes keeps the
-// next ones in flight with cp.async) and adds it, once, into every output
-// plane it touches: input plane ip contributes its 2-D slice w(oz, ., .) to
-// output plane ip - R - oz for oz in [-R, R], so each thread keeps the partial
-// sums of its 4 columns x RPT rows for 2R+1 output planes in registers
+// A work item is a tile of nq quads (16 bytes) x ns TY rows and a run of cz
+// output planes; thread (strip, quad) = (tid / nq, tid mod nq) owns TY rows of
+// four columns.  nq and ns are chosen per grid so that whole tiles cover it with
+// few idle threads (rot_tile).  The CTA stages one input plane at a time (a ring
+// of kRotNPL planes keeps the next ones in flight with cp.async) and adds it,
+// once, into every output plane it touches: input plane ip contributes its 2-D
+// slice w(oz, ., .) to output plane ip - R - oz for oz in [-R, R], so each
+// thread keeps partial sums of its outputs for 2R+1 output planes in registers
 // (slots rotate with the plane index; the plane loop is unrolled by 2R+1, so
 // every slot and weight index is a compile-time constant).  Output plane oq
 // is complete after input plane oq + 2R and is stored from its slot.  Input
 // planes of the first and last 2R of a run also add into slots of outputs
 // outside the run; those slots are cleared, never stored.
-// Staged planes hold columns X0 - 4 .. X0 + 67 (tiles start R mod 4 columns
-// left of the interior, so the window and every thread's 4 output columns
-// are 16-byte aligned): a thread's taps need the 16-byte chunks tx, tx+1,
-// tx+2 of a row; rows that only the centre column touches (star stencils)
-// need chunk tx+1 alone.  Each staged value is read from shared memory once
-// per (row, thread) instead of once per output plane.
+// Staged planes hold quads -1 .. nq of the tile's rows -R .. ns TY + R - 1 (tiles
+// start at a stored column that is a multiple of 4): a thread's taps need the
+// quads qx, qx+1, qx+2 of a staged row; rows that only the centre column touches
+// (star stencils) need quad qx+1 alone.  The quads a thread copies sit at the
+// same place of every plane, so their offsets and masks are found once per
+// item: a copy is one address add and one cp.async (four words where stored
+// rows are not 16-byte multiples).  One barrier per plane.  Word rows are stored
+// through shared memory as coalesced words.
+// Measured, one sweep (64 x 32 tiles, per-copy index arithmetic, two barriers per
+// plane before): Star-3D2R 512^3 305 -> 230 us (HBM floor 159), Box-3D1R
+// 301 x 417 x 533 (words) 240 -> 179 us (floor 80); bound by issue: 27 FMAs of
+// ~40 instructions per output for the box.
 constexpr int kRotNPL = 4;   // ring planes: the one computed and three in flight
-constexpr int kRotPW = 72;   // staged columns (64 + 2 x 4)
+constexpr int kRotCopies = 6;  // quads of a staged plane a thread copies, at most
 
 template <int SHAPE, int R>
 __host__ __device__ constexpr int rot_rows_per_thread()
 {
-    return R <= 2 ? 2 : 1;
-}
-
-template <int SHAPE, int R>
-__host__ __device__ constexpr size_t rot_smem_bytes()
-{
-    return (size_t)kRotNPL * (16 * rot_rows_per_thread<SHAPE, R>() + 2 * R) * kRotPW * sizeof(float);
+    return R == 1 ? 4 : 2;
 }
 
 // Does staged row j (0 .. RPT + 2R - 1) of a thread need more than the
-// centre chunk?  (Yes if some output row i takes it as its own row, oy = 0,
+// centre quad?  (Yes if some output row i takes it as its own row, oy = 0,
 // or the stencil is a box.)
 template <int SHAPE, int R, int RPT>
 __host__ __device__ constexpr bool rot_full_row(int j)
@@ -1285,166 +1287,224 @@ __host__ __device__ constexpr bool rot_full_row(int j)
     return SHAPE == 0 || (j >= R && j < R + RPT);
 }
 
-template <int SHAPE, int R>
-__global__ void __launch_bounds__(kThreads, 2)  // 2 CTAs per SM: the unrolled planes take 80-115 registers
+struct RotTile {
+    int nq = 0, ns = 0;            // quads per row, strips of TY rows
+    int tiles_x = 0, tiles_y = 0;
+    size_t smem = 0;
+};
+
+// The tile of a grid with ny x nx interior points per plane (columns xb .. from
+// the first quad on): the fewest thread-planes, with the staged halo's extra
+// reads weighted by half.
+template <int R, int TY>
+inline RotTile rot_tile(int64_t ny, int64_t span, bool vec)
+{
+    RotTile best;
+    double best_cost = 0;
+    for (int nq = 8; nq <= 64; nq++) {
+        RotTile t;
+        t.nq = nq;
+        t.ns = kThreads / nq;
+        const int ph = t.ns * TY + 2 * R, quads = ph * (nq + 2);
+        if (quads > kRotCopies * kThreads) continue;
+        const int64_t tx = (span + 4 * nq - 1) / (4 * nq), ty = (ny + t.ns * TY - 1) / (t.ns * TY);
+        const double halo = (double)quads / (t.ns * TY * nq);
+        const double cost = (double)tx * ty * (1.0 + 0.5 * (halo - 1.0));
+        if (best.nq == 0 || cost < best_cost) {
+            t.tiles_x = (int)tx;
+            t.tiles_y = (int)ty;
+            t.smem = (size_t)kRotNPL * quads * 16 + (vec ? 0 : kThreads * 16);
+            best = t;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+template <int SHAPE, int R, bool VEC>
+__global__ void __launch_bounds__(kThreads, 2)
     cu3d_rot(const float *__restrict__ in, float *__restrict__ out,
              const __grid_constant__ Weights<float, Taps<SHAPE, 3, R>::K> wt, int64_t Ez, int64_t Ey, int64_t Ex,
-             int tiles_x, int tiles_y, int nitems, int cz, int xs)
+             int nq, int ns, int tiles_x, int tiles_y, int nitems, int cz, int xb)
 {
-    constexpr int RPT = rot_rows_per_thread<SHAPE, R>(), BY = 16 * RPT, BX = 64;
-    constexpr int PH = BY + 2 * R, PW = kRotPW, PE = PH * PW, NS = 2 * R + 1;
-    constexpr int NCH = PW / 4;  // 16-byte chunks per staged row
-    static_assert(R <= 3, "the plane loop unrolls (2R+1)-fold: radii up to 3");
+    constexpr int TY = rot_rows_per_thread<SHAPE, R>(), NS = 2 * R + 1, NPL = kRotNPL;
+    static_assert(R <= 3, "one quad of halo columns per side");
     extern __shared__ __align__(16) float ring[];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int64_t nz = Ez - 2 * R, ny = Ey - 2 * R, nx = Ex - 2 * R;
-    const bool vec = (Ex & 3) == 0 && (reinterpret_cast<uintptr_t>(in) & 15) == 0;
-    const bool vst = (Ex & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    const int tid = threadIdx.x, strip = tid / nq, qx = tid - strip * nq;
+    const bool active = strip < ns;
+    const int PH = ns * TY + 2 * R, PQ = nq + 2, PW = 4 * PQ, quads = PH * PQ, PE = 4 * quads;
+    float *const turn = ring + (size_t)NPL * PE + (tid >> 5) * 128;  // word rows: a warp's 32 quads
+    const int64_t nz = Ez - 2 * R, ny = Ey - 2 * R, nx = Ex - 2 * R, plane = Ey * Ex;
+    const int ex32 = (int)Ex;  // a stored row holds < 2^31 values, and a stored plane too
 
     for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
         const int bx = item % tiles_x, by = (item / tiles_x) % tiles_y, bz = item / (tiles_x * tiles_y);
         // stored coordinates of the item's first output (column X0 may lie in the halo)
-        const int64_t Z0 = R + (int64_t)bz * cz, Y0 = R + (int64_t)by * BY, X0 = R + (int64_t)bx * BX - xs;
+        const int64_t Z0 = R + (int64_t)bz * cz, Y0 = R + (int64_t)by * (ns * TY), X0 = xb + (int64_t)bx * (4 * nq);
         const int64_t rem = nz - (Z0 - R);
         const int nzo = (int)(rem < cz ? rem : cz);
         const int nin = nzo + 2 * R;
-        const int64_t zfirst = Z0 - R;
-        // items whose staged rows and columns lie inside the stored plane (all
-        // but the edges): 32-bit in-plane offsets, no per-chunk tests
-        const bool inner = vec && Y0 - R >= 0 && Y0 - R + PH <= Ey && X0 - 4 >= 0 && X0 - 4 + PW <= Ex;
-        const int ex32 = (int)Ex;                        // a stored row holds < 2^31 values
-        const int base_off = (int)((Y0 - R) * Ex + (X0 - 4));  // and a stored plane too
-        auto load_plane = [&](int ip) {
-            float *dst = ring + (size_t)(ip & (kRotNPL - 1)) * PE;
-            const int64_t gz = zfirst + ip;
-            const bool zok = gz >= 0 && gz < Ez;
-            if (inner && zok) {
-                const float *src = in + gz * Ey * Ex + base_off;
-                for (int e = tid; e < PH * NCH; e += kThreads) {
-                    const int row = e / NCH, ch = e - (e / NCH) * NCH;
-                    cp_async_elem<16>(dst + row * PW + 4 * ch, src + row * ex32 + 4 * ch, true);
-                }
-                return;
+        // this thread's copies: offset within a plane, and which values exist
+        int goff[kRotCopies];
+        unsigned have = 0;  // VEC: bit m; words: bits 4m .. 4m + 3
+#pragma unroll
+        for (int m = 0; m < kRotCopies; ++m) {
+            const int e = tid + m * kThreads, row = e / PQ, ch = e - row * PQ;
+            const int64_t gy = Y0 - R + row, gx = X0 - 4 + 4 * ch;
+            const bool rok = e < quads && gy >= 0 && gy < Ey;
+            goff[m] = rok ? (int)(gy * Ex + gx) : 0;
+            if constexpr (VEC) {
+                have |= (rok && gx >= 0 && gx < Ex) ? 1u << m : 0u;
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) have |= (rok && gx + c >= 0 && gx + c < Ex) ? 1u << (4 * m + c) : 0u;
             }
-            for (int e = tid; e < PH * NCH; e += kThreads) {
-                const int row = e / NCH, ch = e - (e / NCH) * NCH;
-                const int64_t gy = Y0 - R + row, gx = X0 - 4 + 4 * ch;
-                const bool rok = zok && gy >= 0 && gy < Ey;
-                const float *src = in + ((rok ? gz : 0) * Ey + (rok ? gy : 0)) * Ex;
-                float *d = dst + row * PW + 4 * ch;
-                if (vec) {
-                    // gx is a multiple of 4 and so is Ex: the chunk is wholly in or out
-                    const bool ok = rok && gx >= 0 && gx < Ex;
-                    cp_async_elem<16>(d, ok ? src + gx : in, ok);
+        }
+        const float *src = in + (Z0 - R) * plane;  // the next plane to copy
+        auto load_plane = [&](int ip) {
+            float *dst = ring + (size_t)(ip & (NPL - 1)) * PE + 4 * tid;
+#pragma unroll
+            for (int m = 0; m < kRotCopies; ++m) {
+                if (tid + m * kThreads >= quads) break;
+                float *d = dst + 4 * m * kThreads;
+                if constexpr (VEC) {
+                    const bool ok = (have >> m) & 1u;
+                    cp_async_elem<16>(d, ok ? src + goff[m] : in, ok);
                 } else {
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        const bool ok = rok && gx + c >= 0 && gx + c < Ex;
-                        cp_async_elem<4>(d + c, ok ? src + gx + c : in, ok);
+                        const bool ok = (have >> (4 * m + c)) & 1u;
+                        cp_async_elem<4>(d + c, ok ? src + goff[m] + c : in, ok);
                     }
                 }
             }
+            src += plane;
         };
         __syncthreads();  // the previous item's reads of the ring are done
 #pragma unroll
-        for (int k = 0; k < kRotNPL - 1; ++k) {
+        for (int k = 0; k < NPL - 1; ++k) {
             if (k < nin) load_plane(k);
             cp_async_commit();
         }
-        float acc[NS][RPT][4];
+        float acc[NS][TY][4];
 #pragma unroll
         for (int s = 0; s < NS; ++s)
 #pragma unroll
-            for (int i = 0; i < RPT; ++i) acc[s][i][0] = acc[s][i][1] = acc[s][i][2] = acc[s][i][3] = 0.0f;
-        const int64_t gy0 = Y0 + ty * RPT, gx0 = X0 + 4 * tx;
-        // this thread's output quads: offset within a stored plane, row inside
-        // the interior, and which columns are interior
-        const bool qfull = gx0 >= R && gx0 + 3 - R < nx;
-        unsigned cmask = 0;
+            for (int i = 0; i < TY; ++i) acc[s][i][0] = acc[s][i][1] = acc[s][i][2] = acc[s][i][3] = 0.0f;
+        // stores.  VEC: the thread's own quads; words: value j of the warp's 128 is
+        // component lane % 4 of the quad of lane 8 j + lane / 4
+        const int64_t gy0 = Y0 + strip * TY, gx0 = X0 + 4 * qx;
+        const int nrow_ok = active ? (int)min((int64_t)TY, ny + R - gy0) : 0;  // rows of the thread inside the interior
+        unsigned cmask = 0;  // interior columns of the quad
 #pragma unroll
         for (int c = 0; c < 4; ++c) cmask |= (gx0 + c >= R && gx0 + c - R < nx) ? (1u << c) : 0u;
-        const int nrow_ok = (int)min((int64_t)RPT, ny + R - gy0);  // rows of the thread inside the interior
-        const int ooff0 = (int)(gy0 * Ex + gx0);                  // offset within a stored plane
+        float *dst = out + Z0 * plane + gy0 * Ex + gx0;  // the next output plane
+        int woff[VEC ? 1 : 4];   // words: offset of value j from `out`'s plane, rows it is stored in
+        int wrow = 0;  // four bits per j
+        if constexpr (!VEC) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int t2 = (tid & ~31) + 8 * j + ((tid & 31) >> 2), s2 = t2 / nq, q2 = t2 - s2 * nq;
+                const int64_t y2 = Y0 + s2 * TY, x2 = X0 + 4 * q2 + (tid & 3);
+                woff[j] = (int)(y2 * Ex + x2);
+                wrow |= (s2 < ns && x2 >= R && x2 - R < nx ? (int)max((int64_t)0, min((int64_t)TY, ny + R - y2)) : 0)
+                        << (4 * j);
+            }
+            dst = out + Z0 * plane;
+        }
+        const int col = (strip * TY) * PW + 4 * qx;
         for (int base = 0; base < nin; base += NS) {
             // the NS planes of this round; u is a compile-time constant, so every
             // accumulator slot index below is one too (no run-time selects)
-            static_for<NS>([&](auto U) -> bool {
-                constexpr int u = decltype(U)::value;
+            static_for<NS>([&](auto UC) -> bool {
+                constexpr int u = decltype(UC)::value;
                 const int ip = base + u;
                 if (ip >= nin) return false;
-                // plane ip + NPL - 1 goes into the slot plane ip - 1 used (read before the last barrier)
-                if (ip + kRotNPL - 1 < nin) load_plane(ip + kRotNPL - 1);
+                cp_async_wait_group<NPL - 2>();  // this thread's copies of plane ip have landed
+                __syncthreads();                 // everyone's have, and plane ip - 1 is read
+                if (ip + NPL - 1 < nin) load_plane(ip + NPL - 1);
                 cp_async_commit();
-                cp_async_wait_group<kRotNPL - 1>();  // plane ip has landed
-                __syncthreads();
-                const float *pl = ring + (size_t)(ip & (kRotNPL - 1)) * PE + (ty * RPT) * PW + 4 * tx;
+                if (active) {
+                    const float *pl = ring + (size_t)(ip & (NPL - 1)) * PE + col;
 #pragma unroll
-                for (int j = 0; j < RPT + 2 * R; ++j) {
-                    const float *rowp = pl + j * PW;
-                    float v[12];
-                    const float4 c1 = *reinterpret_cast<const float4 *>(rowp + 4);
-                    v[4] = c1.x;
-                    v[5] = c1.y;
-                    v[6] = c1.z;
-                    v[7] = c1.w;
-                    if (rot_full_row<SHAPE, R, RPT>(j)) {
-                        const float4 c0 = *reinterpret_cast<const float4 *>(rowp);
-                        const float4 c2 = *reinterpret_cast<const float4 *>(rowp + 8);
-                        v[0] = c0.x;
-                        v[1] = c0.y;
-                        v[2] = c0.z;
-                        v[3] = c0.w;
-                        v[8] = c2.x;
-                        v[9] = c2.y;
-                        v[10] = c2.z;
-                        v[11] = c2.w;
-                    }
+                    for (int j = 0; j < TY + 2 * R; ++j) {
+                        const float *rowp = pl + j * PW;
+                        float v[12];
+                        const float4 c1 = *reinterpret_cast<const float4 *>(rowp + 4);
+                        v[4] = c1.x;
+                        v[5] = c1.y;
+                        v[6] = c1.z;
+                        v[7] = c1.w;
+                        if (rot_full_row<SHAPE, R, TY>(j)) {
+                            const float4 c0 = *reinterpret_cast<const float4 *>(rowp);
+                            const float4 c2 = *reinterpret_cast<const float4 *>(rowp + 8);
+                            v[0] = c0.x;
+                            v[1] = c0.y;
+                            v[2] = c0.z;
+                            v[3] = c0.w;
+                            v[8] = c2.x;
+                            v[9] = c2.y;
+                            v[10] = c2.z;
+                            v[11] = c2.w;
+                        }
 #pragma unroll
-                    for (int i = 0; i < RPT; ++i) {
-                        const int oy = j - i - R;
-                        if (oy < -R || oy > R) continue;
+                        for (int i = 0; i < TY; ++i) {
+                            const int oy = j - i - R;
+                            if (oy < -R || oy > R) continue;
 #pragma unroll
-                        for (int oz = -R; oz <= R; ++oz) {
-                            const int slot = ((u - R - oz) % NS + 2 * NS) % NS;
+                            for (int oz = -R; oz <= R; ++oz) {
+                                const int slot = ((u - R - oz) % NS + 2 * NS) % NS;
 #pragma unroll
-                            for (int ox = -R; ox <= R; ++ox) {
-                                const int k = tap_index<SHAPE, 3, R>(oz, oy, ox);
-                                if (k >= 0) {
+                                for (int ox = -R; ox <= R; ++ox) {
+                                    const int k = tap_index<SHAPE, 3, R>(oz, oy, ox);
+                                    if (k >= 0) {
 #pragma unroll
-                                    for (int c = 0; c < 4; ++c)
-                                        acc[slot][i][c] = fmaf(wt.w[k], v[4 + c + ox], acc[slot][i][c]);
+                                        for (int c = 0; c < 4; ++c)
+                                            acc[slot][i][c] = fmaf(wt.w[k], v[4 + c + ox], acc[slot][i][c]);
+                                    }
                                 }
                             }
                         }
                     }
                 }
                 // output plane ip - 2R is complete (slot (u + 1) mod NS)
-                const int oq = ip - 2 * R;
                 constexpr int sd = (u + 1) % NS;
-                if (oq >= 0 && oq < nzo) {
-                    float *obase = out + (Z0 + oq) * Ey * Ex;
+                if (ip >= 2 * R) {
 #pragma unroll
-                    for (int i = 0; i < RPT; ++i) {
-                        if (i >= nrow_ok) continue;
-                        float *o = obase + ooff0 + i * ex32;
-                        if (vst && qfull) {
-                            *reinterpret_cast<float4 *>(o) =
-                                make_float4(acc[sd][i][0], acc[sd][i][1], acc[sd][i][2], acc[sd][i][3]);
+                    for (int i = 0; i < TY; ++i) {
+                        if constexpr (VEC) {
+                            if (i < nrow_ok) {
+                                float *o = dst + i * ex32;
+                                if (cmask == 0xfu) {
+                                    *reinterpret_cast<float4 *>(o) =
+                                        make_float4(acc[sd][i][0], acc[sd][i][1], acc[sd][i][2], acc[sd][i][3]);
+                                } else {
+#pragma unroll
+                                    for (int c = 0; c < 4; ++c)
+                                        if ((cmask >> c) & 1u) o[c] = acc[sd][i][c];
+                                }
+                            }
                         } else {
+                            __syncwarp();
+                            *reinterpret_cast<float4 *>(turn + 4 * (tid & 31)) =
+                                make_float4(acc[sd][i][0], acc[sd][i][1], acc[sd][i][2], acc[sd][i][3]);
+                            __syncwarp();
 #pragma unroll
-                            for (int c = 0; c < 4; ++c)
-                                if ((cmask >> c) & 1u) o[c] = acc[sd][i][c];
+                            for (int j = 0; j < 4; ++j) {
+                                const float w = turn[32 * j + (tid & 31)];
+                                if (i < ((wrow >> (4 * j)) & 15)) dst[woff[j] + i * ex32] = w;
+                            }
                         }
                     }
+                    dst += plane;
                 }
 #pragma unroll
-                for (int i = 0; i < RPT; ++i) acc[sd][i][0] = acc[sd][i][1] = acc[sd][i][2] = acc[sd][i][3] = 0.0f;
-                __syncthreads();  // the slot of plane ip is free for plane ip + NPL
+                for (int i = 0; i < TY; ++i) acc[sd][i][0] = acc[sd][i][1] = acc[sd][i][2] = acc[sd][i][3] = 0.0f;
                 return true;
             });
         }
+        cp_async_wait_group<0>();
     }
-    cp_async_wait_group<0>();
 }
 
 }  // namespace cu

@@ -166,30 +166,34 @@ stencil_status launch3d_stream(const Plan &p, const void *in, void *out, cudaStr
 
 // 3-D, t = 1, FP32: z-marching with rotating partial sums (cu3d_rot).  The
 // run of output planes per work item, cz, is chosen so that the items fill
-// whole rounds of the resident CTAs: the time is ~ rounds x (cz + 2R) planes.
-template <int SHAPE, int R>
+// whole rounds of the resident CTAs: the time is ~ rounds x (cz + 2R + a
+// start-up of ~4 planes).
+template <int SHAPE, int R, bool VEC>
 stencil_status launch3d_rot(const Plan &p, const void *in, void *out, cudaStream_t st)
 {
     using Wt = cu::Weights<float, cu::Taps<SHAPE, 3, R>::K>;
     Wt wt;
     for (int k = 0; k < cu::Taps<SHAPE, 3, R>::K; k++) wt.w[k] = (float)p.w[k];
-    const size_t smem = cu::rot_smem_bytes<SHAPE, R>();
-    auto kern = cu::cu3d_rot<SHAPE, R>;
-    stencil_status s = ensure_smem((const void *)kern, smem);
+    const int xb = R - R % 4;  // the first tile's first column: a multiple of 4
+    const cu::RotTile tile =
+        cu::rot_tile<R, cu::rot_rows_per_thread<SHAPE, R>()>(p.dims[1], p.dims[2] + R - xb, VEC);
+    if (tile.nq == 0 || tile.smem > kMaxSmem)
+        return fail(STENCIL_ERR_UNSUPPORTED, "3-D marching tile does not fit in shared memory");
+    auto kern = cu::cu3d_rot<SHAPE, R, VEC>;
+    stencil_status s = ensure_smem((const void *)kern, tile.smem);
     if (s != STENCIL_OK) return s;
     int occ = 0;
-    s = occupancy((const void *)kern, cu::kThreads, smem, &occ);
+    s = occupancy((const void *)kern, cu::kThreads, tile.smem, &occ);
     if (s != STENCIL_OK) return s;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int BY = 16 * cu::rot_rows_per_thread<SHAPE, R>(), BX = 64, xs = R % 4;
-    const int64_t nz = p.dims[0], tyy = (p.dims[1] + BY - 1) / BY, txx = (p.dims[2] + xs + BX - 1) / BX;
-    const int64_t cols = tyy * txx, slots = (int64_t)std::max(1, occ) * std::max(1, sms);
+    const int64_t nz = p.dims[0], cols = (int64_t)tile.tiles_x * tile.tiles_y;
+    const int64_t slots = (int64_t)std::max(1, occ) * std::max(1, sms);
     int64_t cz = nz, best = -1;
     for (int64_t m = 1; m <= std::min<int64_t>(nz, 512); m++) {
         const int64_t c = (nz + m - 1) / m, items = ((nz + c - 1) / c) * cols;
-        const int64_t cost = (items + slots - 1) / slots * (c + 2 * R);
+        const int64_t cost = (items + slots - 1) / slots * (c + 2 * R + 4);
         if (best < 0 || cost < best) {
             best = cost;
             cz = c;
@@ -198,8 +202,8 @@ stencil_status launch3d_rot(const Plan &p, const void *in, void *out, cudaStream
     const int64_t items = ((nz + cz - 1) / cz) * cols;
     if (items > 0x7fffffff || cz > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const unsigned grid = (unsigned)std::min<int64_t>(items, slots);
-    kern<<<grid, cu::kThreads, smem, st>>>((const float *)in, (float *)out, wt, p.ext[0], p.ext[1], p.ext[2],
-                                           (int)txx, (int)tyy, (int)items, (int)cz, xs);
+    kern<<<grid, cu::kThreads, tile.smem, st>>>((const float *)in, (float *)out, wt, p.ext[0], p.ext[1], p.ext[2],
+                                                tile.nq, tile.ns, tile.tiles_x, tile.tiles_y, (int)items, (int)cz, xb);
     note_launch();
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu3d_rot launch");
@@ -211,7 +215,10 @@ stencil_status launch3d(const Plan &p, const void *in, void *out, int t, cudaStr
     if (t == 1) {
         // FP32 star r <= 3 and box r = 1: rotating partial sums; the rest streams
         if constexpr (sizeof(T) == 4 && ((SHAPE == 1 && R <= 3) || (SHAPE == 0 && R == 1)))
-            return launch3d_rot<SHAPE, R>(p, in, out, st);
+            return p.ext[2] % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0 &&
+                           reinterpret_cast<uintptr_t>(out) % 16 == 0
+                       ? launch3d_rot<SHAPE, R, true>(p, in, out, st)
+                       : launch3d_rot<SHAPE, R, false>(p, in, out, st);
         return launch3d_stream<T, SHAPE, R>(p, in, out, st);
     }
     using Wt = cu::Weights<T, cu::Taps<SHAPE, 3, R>::K>;
