@@ -718,6 +718,14 @@ constexpr int kMarchThreads = 256;
 
 constexpr int kMarchDepth = 8;  // ring rows per warp (a power of two)
 
+// The (shape, radius, depth) triples built: depth 2 where the partial sums and
+// weights of two steps fit in registers.
+template <int SHAPE, int R, int T>
+__host__ __device__ constexpr bool march_has()
+{
+    return R <= 3 && (T == 1 || (T == 2 && (R == 1 || (SHAPE == 1 && R <= 3))));
+}
+
 // Columns a warp yields.
 template <int R, int T>
 __host__ __device__ constexpr int march_cols()
@@ -732,156 +740,173 @@ __host__ __device__ constexpr int march_ctas()
     return T == 1 ? (R <= 2 ? 3 : 2) : 2;  // K weights and 4 T (2R + 1) partial sums in registers
 }
 
+// Floats of shared memory per warp: the ring of input rows and (words only) a
+// row on its way out.
+template <bool VEC>
+__host__ __device__ constexpr int march_warp_floats()
+{
+    return 128 * (kMarchDepth + (VEC ? 0 : 1));
+}
+
+// One work item of a warp: output rows [y0, y1), the cw <= march_cols columns
+// from w0 + 4T on (w0: first column of the 128-column window, a multiple of 4 where VEC).
+template <int SHAPE, int R, int T, bool VEC, typename WT>
+__device__ __forceinline__ void march_strip(const float *__restrict__ in, float *__restrict__ out, const WT &wt,
+                                            int64_t Ey, int64_t Ex, int64_t w0, int64_t y0, int64_t y1, int cw,
+                                            float *ring)
+{
+    constexpr int NS = 2 * R + 1, U = NS, D = kMarchDepth;
+    static_assert(R >= 1 && R <= 4, "one quad of halo columns per side and step");
+    float *const turn_out = ring + 128 * D;
+    const int lane = threadIdx.x & 31;
+    const int64_t x = w0 + 4 * lane;  // this lane's columns x .. x + 3
+    const int64_t ys = y0 - R * T;  // first input row
+    const int nrows = (int)(y1 - y0) + 2 * R * T;
+    // interior columns of the quad, and columns this lane stores
+    unsigned cint = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) cint |= (x + c >= R && x + c < Ex - R) ? 1u << c : 0u;
+    const bool store_lane = lane >= T && lane < T + cw / 4;
+    const bool xok = x >= 0 && x < Ex;  // VEC: a quad lies wholly inside or outside a row
+    // rows i that exist and are wanted: [i_lo, i_hi)
+    const int i_lo = ys < 0 ? (int)-ys : 0, i_hi = (int)min((int64_t)nrows, Ey - ys);
+    float *o = out + (ys - R * T) * Ex + (VEC ? x : w0 + lane);  // the row completed after input row i
+    const float *src = in + ys * Ex + (VEC ? x : w0 + lane);
+    // copy input row ys + i to its ring row (rows and columns outside the stored array become zero)
+    auto load = [&](int i) {
+        const bool rok = i >= i_lo && i < i_hi;
+        float *d = ring + (i & (D - 1)) * 128 + (VEC ? 4 * lane : lane);
+        if constexpr (VEC) {
+            const bool ok = rok && xok;
+            cp_async_elem<16>(d, ok ? src : in, ok);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t gx = w0 + lane + 32 * j;
+                const bool ok = rok && gx >= 0 && gx < Ex;
+                cp_async_elem<4>(d + 32 * j, ok ? src + 32 * j : in, ok);
+            }
+        }
+        cp_async_commit();
+        src += Ex;
+    };
+    cp_async_wait_group<0>();  // the previous item's rows have landed and are read
+    __syncwarp();
+    for (int i = 0; i < D - 1; ++i) load(i);
+    float acc[T][NS][4];
+#pragma unroll
+    for (int s = 0; s < T; ++s)
+#pragma unroll
+        for (int m = 0; m < NS; ++m) acc[s][m][0] = acc[s][m][1] = acc[s][m][2] = acc[s][m][3] = 0.0f;
+    // values of the rows R back, which the fixed boundary keeps (t > 1)
+    float hist[T > 1 ? T - 1 : 1][NS][4];
+    for (int base = 0; base < nrows; base += U) {
+        static_for<U>([&](auto UC) -> bool {
+            constexpr int u = decltype(UC)::value;
+            const int i = base + u;
+            if (i >= nrows) return false;
+            cp_async_wait_group<D - 2>();  // row i has landed
+            if constexpr (!VEC) __syncwarp();
+            float q[4];
+            {
+                const float4 t4 = *reinterpret_cast<const float4 *>(ring + (i & (D - 1)) * 128 + 4 * lane);
+                q[0] = t4.x;
+                q[1] = t4.y;
+                q[2] = t4.z;
+                q[3] = t4.w;
+            }
+            // row i + D - 1 takes the ring row of row i - 1, whose quads every lane has read
+            load(i + D - 1);
+            static_for<T>([&](auto SC) -> bool {
+                constexpr int s = decltype(SC)::value;   // fused step s + 1; its input row is ys + i - s R
+                constexpr int us = ((u - 2 * R * s) % NS + NS) % NS;  // that row's slot phase
+                if (s > 0 && i < 2 * R * s) return false;  // no complete row of step s yet
+                float v[4 + 2 * R];
+#pragma unroll
+                for (int c = 0; c < R; ++c) {
+                    v[c] = __shfl_up_sync(0xffffffffu, q[4 - R + c], 1);
+                    v[R + 4 + c] = __shfl_down_sync(0xffffffffu, q[c], 1);
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[R + c] = q[c];
+                if constexpr (s < T - 1) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) hist[s][us][c] = q[c];
+                }
+                // row j (relative) adds into outputs j - e, e = 0 .. 2R, with oy = e - R
+#pragma unroll
+                for (int e = 0; e < NS; ++e) {
+                    const int slot = ((us - e) % NS + NS) % NS;
+#pragma unroll
+                    for (int ox = -R; ox <= R; ++ox) {
+                        const int k = tap_index<SHAPE, 2, R>(0, e - R, ox);
+                        if (k >= 0) {
+#pragma unroll
+                            for (int c = 0; c < 4; ++c)
+                                acc[s][slot][c] = fmaf(wt.w[k], v[R + ox + c], acc[s][slot][c]);
+                        }
+                    }
+                }
+                // output j - 2R is complete: slot (us + 1) mod NS
+                constexpr int done = (us + 1) % NS;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    q[c] = acc[s][done][c];
+                    acc[s][done][c] = 0.0f;
+                }
+                if constexpr (s < T - 1) {
+                    // the halo keeps its value between the fused steps
+                    const int64_t y = ys + i - (int64_t)R * (s + 1);  // the completed row
+                    const bool rint = y >= R && y < Ey - R;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (!(rint && ((cint >> c) & 1u))) q[c] = hist[s][((us - R) % NS + NS) % NS][c];
+                } else if (i >= 2 * R * T) {
+                    if constexpr (VEC) {
+                        if (store_lane) {
+                            if (cint == 0xfu) {
+                                *reinterpret_cast<float4 *>(o) = make_float4(q[0], q[1], q[2], q[3]);
+                            } else {
+#pragma unroll
+                                for (int c = 0; c < 4; ++c)
+                                    if ((cint >> c) & 1u) o[c] = q[c];
+                            }
+                        }
+                    } else {
+                        *reinterpret_cast<float4 *>(turn_out + 4 * lane) = make_float4(q[0], q[1], q[2], q[3]);
+                        __syncwarp();
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int col = 32 * j + lane;
+                            const int64_t gx = w0 + col;
+                            if (col >= 4 * T && col < 4 * T + cw && gx >= R && gx < Ex - R)
+                                o[32 * j] = turn_out[col];
+                        }
+                        __syncwarp();
+                    }
+                }
+                return true;
+            });
+            o += Ex;
+            return true;
+        });
+    }
+}
+
 template <int SHAPE, int R, int T, bool VEC>
 __global__ void __launch_bounds__(kMarchThreads, (march_ctas<SHAPE, R, T>()))
     cu2d_march(const float *__restrict__ in, float *__restrict__ out,
                const __grid_constant__ Weights<float, Taps<SHAPE, 2, R>::K> wt, int64_t Ey, int64_t Ex, int ncb,
                int seg, int nitems, int xb)
 {
-    constexpr int NS = 2 * R + 1, U = NS, CW = march_cols<R, T>(), D = kMarchDepth;
-    static_assert(R >= 1 && R <= 4, "one quad of halo columns per side and step");
-    // per warp: the ring of input rows and (words only) a row on its way out
-    __shared__ __align__(16) float smem[(kMarchThreads / 32) * 128 * (D + (VEC ? 0 : 1))];
-    const int lane = threadIdx.x & 31;
-    float *const ring = smem + (threadIdx.x >> 5) * 128 * (D + (VEC ? 0 : 1)), *const turn_out = ring + 128 * D;
+    constexpr int CW = march_cols<R, T>();
+    __shared__ __align__(16) float smem[(kMarchThreads / 32) * march_warp_floats<VEC>()];
+    float *const ring = smem + (threadIdx.x >> 5) * march_warp_floats<VEC>();
     const int nwarps = (int)(gridDim.x * (kMarchThreads / 32));
     for (int item = (int)(blockIdx.x * (kMarchThreads / 32) + (threadIdx.x >> 5)); item < nitems; item += nwarps) {
-        const int cb = item % ncb;
-        const int64_t y0 = R + (int64_t)(item / ncb) * seg;        // first output row
-        const int64_t y1 = min(y0 + seg, Ey - R);                  // end of the output rows
-        const int64_t w0 = xb + (int64_t)cb * CW - 4 * T;          // first column of the window
-        const int64_t x = w0 + 4 * lane;                           // this lane's columns x .. x + 3
-        const int64_t ys = y0 - R * T;                             // first input row
-        const int nrows = (int)(y1 - y0) + 2 * R * T;
-        // interior columns of the quad, and columns this lane stores
-        unsigned cint = 0;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) cint |= (x + c >= R && x + c < Ex - R) ? 1u << c : 0u;
-        const bool store_lane = lane >= T && lane < 32 - T;
-        const bool xok = x >= 0 && x < Ex;  // VEC: a quad lies wholly inside or outside a row
-        // rows i that exist and are wanted: [i_lo, i_hi)
-        const int i_lo = ys < 0 ? (int)-ys : 0, i_hi = (int)min((int64_t)nrows, Ey - ys);
-        float *o = out + (ys - R * T) * Ex + (VEC ? x : w0 + lane);  // the row completed after input row i
-        const float *src = in + ys * Ex + (VEC ? x : w0 + lane);
-        // copy input row ys + i to its ring row (rows and columns outside the stored array become zero)
-        auto load = [&](int i) {
-            const bool rok = i >= i_lo && i < i_hi;
-            float *d = ring + (i & (D - 1)) * 128 + (VEC ? 4 * lane : lane);
-            if constexpr (VEC) {
-                const bool ok = rok && xok;
-                cp_async_elem<16>(d, ok ? src : in, ok);
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int64_t gx = w0 + lane + 32 * j;
-                    const bool ok = rok && gx >= 0 && gx < Ex;
-                    cp_async_elem<4>(d + 32 * j, ok ? src + 32 * j : in, ok);
-                }
-            }
-            cp_async_commit();
-            src += Ex;
-        };
-        cp_async_wait_group<0>();  // the previous item's rows have landed and are read
-        __syncwarp();
-        for (int i = 0; i < D - 1; ++i) load(i);
-        float acc[T][NS][4];
-#pragma unroll
-        for (int s = 0; s < T; ++s)
-#pragma unroll
-            for (int m = 0; m < NS; ++m) acc[s][m][0] = acc[s][m][1] = acc[s][m][2] = acc[s][m][3] = 0.0f;
-        // values of the rows R back, which the fixed boundary keeps (t > 1)
-        float hist[T > 1 ? T - 1 : 1][NS][4];
-        for (int base = 0; base < nrows; base += U) {
-            static_for<U>([&](auto UC) -> bool {
-                constexpr int u = decltype(UC)::value;
-                const int i = base + u;
-                if (i >= nrows) return false;
-                cp_async_wait_group<D - 2>();  // row i has landed
-                if constexpr (!VEC) __syncwarp();
-                float q[4];
-                {
-                    const float4 t4 = *reinterpret_cast<const float4 *>(ring + (i & (D - 1)) * 128 + 4 * lane);
-                    q[0] = t4.x;
-                    q[1] = t4.y;
-                    q[2] = t4.z;
-                    q[3] = t4.w;
-                }
-                // row i + D - 1 takes the ring row of row i - 1, whose quads every lane has read
-                load(i + D - 1);
-                static_for<T>([&](auto SC) -> bool {
-                    constexpr int s = decltype(SC)::value;   // fused step s + 1; its input row is ys + i - s R
-                    constexpr int us = ((u - 2 * R * s) % NS + NS) % NS;  // that row's slot phase
-                    if (s > 0 && i < 2 * R * s) return false;  // no complete row of step s yet
-                    float v[4 + 2 * R];
-#pragma unroll
-                    for (int c = 0; c < R; ++c) {
-                        v[c] = __shfl_up_sync(0xffffffffu, q[4 - R + c], 1);
-                        v[R + 4 + c] = __shfl_down_sync(0xffffffffu, q[c], 1);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) v[R + c] = q[c];
-                    if constexpr (s < T - 1) {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) hist[s][us][c] = q[c];
-                    }
-                    // row j (relative) adds into outputs j - e, e = 0 .. 2R, with oy = e - R
-#pragma unroll
-                    for (int e = 0; e < NS; ++e) {
-                        const int slot = ((us - e) % NS + NS) % NS;
-#pragma unroll
-                        for (int ox = -R; ox <= R; ++ox) {
-                            const int k = tap_index<SHAPE, 2, R>(0, e - R, ox);
-                            if (k >= 0) {
-#pragma unroll
-                                for (int c = 0; c < 4; ++c)
-                                    acc[s][slot][c] = fmaf(wt.w[k], v[R + ox + c], acc[s][slot][c]);
-                            }
-                        }
-                    }
-                    // output j - 2R is complete: slot (us + 1) mod NS
-                    constexpr int done = (us + 1) % NS;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        q[c] = acc[s][done][c];
-                        acc[s][done][c] = 0.0f;
-                    }
-                    if constexpr (s < T - 1) {
-                        // the halo keeps its value between the fused steps
-                        const int64_t y = ys + i - (int64_t)R * (s + 1);  // the completed row
-                        const bool rint = y >= R && y < Ey - R;
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            if (!(rint && ((cint >> c) & 1u))) q[c] = hist[s][((us - R) % NS + NS) % NS][c];
-                    } else if (i >= 2 * R * T) {
-                        if constexpr (VEC) {
-                            if (store_lane) {
-                                if (cint == 0xfu) {
-                                    *reinterpret_cast<float4 *>(o) = make_float4(q[0], q[1], q[2], q[3]);
-                                } else {
-#pragma unroll
-                                    for (int c = 0; c < 4; ++c)
-                                        if ((cint >> c) & 1u) o[c] = q[c];
-                                }
-                            }
-                        } else {
-                            *reinterpret_cast<float4 *>(turn_out + 4 * lane) = make_float4(q[0], q[1], q[2], q[3]);
-                            __syncwarp();
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const int col = 32 * j + lane;
-                                const int64_t gx = w0 + col;
-                                if (col >= 4 * T && col < 128 - 4 * T && gx >= R && gx < Ex - R)
-                                    o[32 * j] = turn_out[col];
-                            }
-                            __syncwarp();
-                        }
-                    }
-                    return true;
-                });
-                o += Ex;
-                return true;
-            });
-        }
+        const int64_t y0 = R + (int64_t)(item / ncb) * seg;
+        march_strip<SHAPE, R, T, VEC>(in, out, wt, Ey, Ex, xb + (int64_t)(item % ncb) * CW - 4 * T, y0,
+                                      min(y0 + seg, Ey - R), CW, ring);
     }
     cp_async_wait_group<0>();
 }

@@ -68,7 +68,7 @@ stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStr
     for (int k = 0; k < cu::Taps<SHAPE, 2, R>::K; k++) wt.w[k] = (T)p.w[k];
     int tile[3] = {p.tile[0], p.tile[1], p.tile[2]};
     if (p.path != STENCIL_PATH_CUDA_CORE) cu_default_tile(p, t, tile);
-    if constexpr (sizeof(T) == 4 && R <= (SHAPE == 0 ? 2 : 3)) {
+    if constexpr (sizeof(T) == 4 && R <= 3) {
         // a tile asked for by option or picked by the autotuner runs the tiled kernel
         int def[3];
         cu_default_tile(p, p.t, def);
@@ -78,8 +78,7 @@ stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStr
             if (t == 1)
                 return vec ? launch2d_march<SHAPE, R, 1, true>(p, in, out, st)
                            : launch2d_march<SHAPE, R, 1, false>(p, in, out, st);
-            // two steps where their partial sums and weights fit in registers
-            if constexpr (R == 1 || (SHAPE == 1 && R == 2))
+            if constexpr (cu::march_has<SHAPE, R, 2>())
                 return vec ? launch2d_march<SHAPE, R, 2, true>(p, in, out, st)
                            : launch2d_march<SHAPE, R, 2, false>(p, in, out, st);
         }

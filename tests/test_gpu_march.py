@@ -80,3 +80,28 @@ def test_same_bits_as_the_tiled_kernel(torch, shape, r, t):
         outs.append(y.cpu().numpy())
         plan.close()
     np.testing.assert_array_equal(outs[0], outs[1])
+
+
+def test_batched_marching_tiles(torch):
+    """The batched kernel's marching path over thin, ragged and aligned grids: the same bits as single runs
+    (remainder sweeps of depth 1 on tiles cut for depth 2 included)."""
+    shapes = [("box", 1), ("box", 2), ("box", 3), ("star", 1), ("star", 2), ("star", 3)]
+    dims = [(1, 1), (3, 300), (300, 2), (64, 119), (65, 241), (130, 448), (257, 700), (1100, 1000)]
+    grids, ins = [], []
+    rng = np.random.default_rng(21)
+    for i, (ny, nx) in enumerate(dims):
+        for shape, r in shapes:
+            grids.append((shape, r, ny, nx, inputs.weights(shape, 2, r, 40 + i)))
+            ins.append(torch.from_numpy(rng.uniform(-1, 1, size=(ny + 2 * r, nx + 2 * r)).astype(np.float32)).cuda())
+    batch = B.Batch(grids, "f32")
+    outs = [torch.full_like(x, float("nan")) for x in ins]
+    for steps in (1, 7):
+        batch.run(ins, outs, steps)
+        B.stencil_batch_status(batch.handle)
+        for (shape, r, ny, nx, w), x, y in zip(grids, ins, outs):
+            plan = B.Plan(shape, 2, r, w, "f32", (ny, nx), 0, path="cuda_core")
+            ref = torch.empty_like(x)
+            plan.run(x, ref, steps)
+            assert torch.equal(y, ref), (shape, r, ny, nx, steps)
+            plan.close()
+    batch.close()
