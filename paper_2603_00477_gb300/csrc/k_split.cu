@@ -49,6 +49,7 @@
 #include <cstdint>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "cu_kernels.cuh"
@@ -243,42 +244,52 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
 
     if (warp == kWorkerWarps) {
-        // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            const uint32_t lbo_a = (uint32_t)HS * 16;
-            const uint64_t db0 = smem_desc(smem_u32(Bm), 128, 256);
-            int k = 0;
-            for (int id = blockIdx.x; id < ntiles; id += gridDim.x, ++k) {
-                const int bf = k & 1;
-                if (!bounded_wait(&full[bf], (k >> 1) & 1, kWaitCycles)) break;
-                if (k >= 2 && !bounded_wait(&freeb[bf], ((k - 2) >> 1) & 1, kWaitCycles)) break;
-                fence_after_thread_sync();
-                const uint64_t da0 = smem_desc(smem_u32(A[bf]), lbo_a, 128);
-                const uint32_t dset = tmem + bf * kSet;
-                uint32_t first = 1;
-                for (int a = 0; a < lines; ++a) {
-                    for (int kb = p.kb_lo[a]; kb <= p.kb_hi[a]; ++kb) {
-                        const uint64_t db = db0 + (uint64_t)((uint32_t)(a * kNkb + kb) * kBlk >> 4);
+        // ---------------- MMA issuer (the whole warp; one elected lane issues) ----------------
+        // Issued by one diverged lane with 64-bit descriptor arithmetic an MMA took ~90 cycles whatever
+        // its N; from a converged warp it takes ~50 (the least; its arithmetic is N / 2 = 48 .. 8).
+        const uint32_t leader = elect_lane();
+        const uint64_t bdesc = smem_desc(smem_u32(Bm), 128, 256);
+        const uint32_t bhi = (uint32_t)(bdesc >> 32), db0 = (uint32_t)bdesc;
+        const uint32_t lbo_a = (uint32_t)HS * 16, slice16 = slice_bytes >> 4;
+        int k = 0;
+        for (int id = blockIdx.x; id < ntiles; id += gridDim.x, ++k) {
+            const int bf = k & 1;
+            bool up = bounded_wait(&full[bf], (k >> 1) & 1, kWaitCycles);
+            if (k >= 2) up = up && bounded_wait(&freeb[bf], ((k - 2) >> 1) & 1, kWaitCycles);
+            if (!__all_sync(0xffffffffu, up)) break;
+            fence_after_thread_sync();
+            const uint64_t adesc = smem_desc(smem_u32(A[bf]), lbo_a, 128);
+            const uint32_t ahi = (uint32_t)(adesc >> 32), da0 = (uint32_t)adesc;
+            const uint32_t dset = tmem + bf * kSet;
+            // one (line, K block): slice i of the input times the weight digits 0 .. S-1-i
+            auto block = [&](auto first, uint32_t da, uint32_t db) {
+                constexpr int ACC0 = decltype(first)::value ? 0 : 1;
 #pragma unroll
-                        for (int i = 0; i < S; ++i) {
-                            const uint32_t idesc = instr_desc(kFmtF16, TM, TN * (S - i));
+                for (int i = 0; i < S; ++i) {
+                    const uint32_t idesc = instr_desc(kFmtF16, TM, TN * (S - i));
 #pragma unroll
-                            for (int q = 0; q < NACC; ++q) {
-                                // A slice i, window of column block q, K block kb, line a
-                                const uint32_t aoff = i * slice_bytes + (uint32_t)((2 * q + 2 * kb) * HS + a) * 16;
-                                mma_f16(dset + (uint32_t)(q * TN * S + TN * i), da0 + (aoff >> 4), db, idesc,
-                                        (first && i == 0) ? 0u : 1u);
-                            }
-                        }
-                        first = 0;
+                    for (int q = 0; q < NACC; ++q) {
+                        const uint32_t d = dset + (uint32_t)(q * TN * S + TN * i);
+                        const uint32_t dai = da + i * slice16 + (uint32_t)(2 * q * HS);
+                        if (i == 0) mma_f16_warp<ACC0>(leader, d, dai, ahi, db, bhi, idesc);
+                        else mma_f16_warp<1>(leader, d, dai, ahi, db, bhi, idesc);
                     }
                 }
-                mma_commit(&done[bf]);
-            }
-            // the last MMAs finish before TMEM can be freed
-            if (k >= 1) wait_cycles(&done[(k - 1) & 1], ((k - 1) >> 1) & 1, kWaitCycles);
-            if (k >= 2) wait_cycles(&done[(k - 2) & 1], ((k - 2) >> 1) & 1, kWaitCycles);
+            };
+            bool first = true;
+            for (int a = 0; a < lines; ++a)
+                for (int kb = p.kb_lo[a]; kb <= p.kb_hi[a]; ++kb) {
+                    const uint32_t da = da0 + (uint32_t)(2 * kb * HS + a);
+                    const uint32_t db = db0 + ((uint32_t)(a * kNkb + kb) * kBlk >> 4);
+                    if (first) block(std::true_type{}, da, db);
+                    else block(std::false_type{}, da, db);
+                    first = false;
+                }
+            mma_commit_warp(leader, &done[bf]);
         }
+        // the last MMAs finish before TMEM can be freed
+        if (k >= 1) wait_cycles(&done[(k - 1) & 1], ((k - 1) >> 1) & 1, kWaitCycles);
+        if (k >= 2) wait_cycles(&done[(k - 2) & 1], ((k - 2) >> 1) & 1, kWaitCycles);
         __syncwarp();
     } else {
         // -------- loaders / digit cutters and epilogue (warps 0-15) --------
