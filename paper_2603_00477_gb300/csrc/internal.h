@@ -85,6 +85,9 @@ struct Plan {
     int tile[3] = {1, 1, 1};
     stencil_info info{};
 
+    // composite kernels w^(t) the tensor-core launchers have used (composite())
+    mutable std::vector<std::vector<double>> composites;
+
     // device workspace (caller owned)
     void *ws = nullptr;
     size_t ws_bytes = 0;
@@ -92,6 +95,12 @@ struct Plan {
     size_t elem_bytes() const { return dtype == STENCIL_F64 ? 8 : 4; }
     size_t grid_bytes() const { return (size_t)n_stored * elem_bytes(); }
 };
+
+// w^(t) of the plan (compose_dense), computed at the first launch of a depth and
+// kept with the plan: at t r = 9 the convolution takes tens of microseconds of
+// host time, more than a small grid's sweep.  Like every use of a plan, one
+// thread at a time.
+const std::vector<double> &composite(const Plan &p, int t);
 
 stencil_status dispatch(Plan *p);  // fills path/precision/t/tile/info
 

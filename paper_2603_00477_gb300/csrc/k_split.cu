@@ -509,7 +509,7 @@ stencil_status split_fill(const Plan &p, int t, split::SplitParams *sp, int *S_o
     if (p.pat.d != 2 || p.dtype != STENCIL_F64)
         return fail(STENCIL_ERR_UNSUPPORTED, "split FP64 path: 2-D FP64 grids only");
     if (R > kMaxR) return fail(STENCIL_ERR_UNSUPPORTED, "split FP64 path: fused radius t*r must be <= 8");
-    const std::vector<double> wt = compose_dense(p.pat, p.w, t);
+    const std::vector<double> &wt = composite(p, t);
     const int lines = 2 * R + 1, taps = lines * lines;
     double wmax = 0;
     for (double x : wt) wmax = std::max(wmax, std::fabs(x));

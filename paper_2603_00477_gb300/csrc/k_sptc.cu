@@ -347,7 +347,7 @@ stencil_status launch_sptc_sweep(const Plan &p, const void *in, void *out, int t
     const SpLayout L = sp_layout_2d(p.pat.shape, r, t);
     SpParams sp;
     std::memset(&sp, 0, sizeof(sp));
-    const std::vector<double> wt = compose_dense(p.pat, p.w, t);
+    const std::vector<double> &wt = composite(p, t);
     const int lines = 2 * R + 1;
     for (int i = 0; i < lines * lines; i++) sp.w[i] = wt[i];
     for (int i = 0; i < 2 * kSpMaxNs; i++) {

@@ -123,7 +123,7 @@ stencil_status fill_params(const Plan &p, int t, int n_tile, int k_inst, TcParam
     const int r = p.pat.r, R = t * r;
     if (R > kTcMaxR) return fail(STENCIL_ERR_UNSUPPORTED, "tensor-core path: fused radius t*r must be <= 12");
     *L = tc_lines_2d(p.pat.shape, r, t, n_tile, k_inst);
-    std::vector<double> wt = compose_dense(p.pat, p.w, t);
+    const std::vector<double> &wt = composite(p, t);
     std::memset(tp, 0, sizeof(*tp));
     const int lines = 2 * R + 1;
     for (int i = 0; i < lines * lines; i++) tp->w[i] = wt[i];

@@ -681,7 +681,7 @@ stencil_status launch_form(const Plan &p, const void *in, void *out, int t, cuda
     if (g.gn == 0) return fail(STENCIL_ERR_UNSUPPORTED, "tensor-core tile does not fit in shared memory");
     WideParams wp;
     std::memset(&wp, 0, sizeof(wp));
-    const std::vector<double> wt = compose_dense(p.pat, p.w, t);
+    const std::vector<double> &wt = composite(p, t);
     const int lines = 2 * R + 1;
     double wmax = 0;
     for (int i = 0; i < lines * lines; i++) {

@@ -492,7 +492,7 @@ stencil_status launch_wide3_n(const Plan &p, const void *in, void *out, cudaStre
         int &h = half[dz + R][dy + R];
         h = std::max(h, std::abs(dx));
     }
-    const std::vector<double> wd = compose_dense(p.pat, p.w, 1);  // (2R+1)^3, (dz, dy, dx) lexicographic
+    const std::vector<double> &wd = composite(p, 1);  // (2R+1)^3, (dz, dy, dx) lexicographic
     Wide3Params wp;
     std::memset(&wp, 0, sizeof(wp));
     const int nkb = (128 + 2 * R + 15) / 16;

@@ -60,6 +60,14 @@ stencil_status abi_exception(const char *entry) noexcept
     return s;
 }
 
+const std::vector<double> &composite(const Plan &p, int t)
+{
+    if (p.composites.size() <= (size_t)t) p.composites.resize(t + 1);
+    std::vector<double> &c = p.composites[t];
+    if (c.empty()) c = compose_dense(p.pat, p.w, t);
+    return c;
+}
+
 void note_launch(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 // Radii the CUDA-core kernels are instantiated for (k_cuda_core*.cu).
