@@ -211,15 +211,24 @@ __global__ void __launch_bounds__(kThreads, 1)
     // j = 0..S-1, rows n' = 16 j + n (output column n) and k = 0..15 of the
     // window, B[n'][k] = b_j(a, kb*16 + k - n - R) in its band; K-major core
     // matrices (n-group g, k-chunk c) at g*256 + c*128.
+    // (Each digit is converted once, into a table where the first operand buffer
+    // will be: indexed straight from the kernel parameters, every lane at its own
+    // address, this took ~20 us of every sweep.)
+    unsigned short *const tab = reinterpret_cast<unsigned short *>(A[0]);
+    for (int idx = tid; idx < S * lines * lines; idx += blockDim.x) {
+        const int j = idx / (lines * lines);
+        tab[idx] = __half_as_ushort(__int2half_rn(p.wd[j][idx - j * lines * lines]));
+    }
+    __syncthreads();
     const int bent = lines * kNkb * TN * S * KI;
     for (int idx = tid; idx < bent; idx += blockDim.x) {
         const int k = idx % KI, nn = (idx / KI) % (TN * S), blk = idx / (KI * TN * S);
         const int a = blk / kNkb, kb = blk % kNkb;
         const int j = nn / TN, n = nn % TN;
         const int c = kb * KI + k - n - R;
-        const int dgt = (c >= -R && c <= R) ? p.wd[j][a * lines + (c + R)] : 0;
+        const unsigned short dgt = (c >= -R && c <= R) ? tab[(j * lines + a) * lines + (c + R)] : (unsigned short)0;
         const uint32_t off = blk * kBlk + (nn / 8) * 256 + (k / 8) * 128 + (nn % 8) * 16 + (k % 8) * 2;
-        *reinterpret_cast<__half *>(Bm + off) = __int2half_rn(dgt);
+        *reinterpret_cast<unsigned short *>(Bm + off) = dgt;
     }
     fence_proxy_async_smem();
     fence_before_thread_sync();

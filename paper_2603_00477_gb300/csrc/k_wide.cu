@@ -249,23 +249,39 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
         for (int s = 0; s < 4; ++s) mbar_init(&eub[s], 1);
         fence_mbar_init();
     }
-    // weight strip: core matrix (L, c), L = ky + g, holds line L - 15
+    // Weight strip: core matrix (L, c), L = ky + g, holds line L - 15.  Each
+    // weight is rounded to its operand parts once (FP64 arithmetic runs at two
+    // lanes per cycle), then the strip is a copy of table entries.
     {
+        uint32_t *const th = reinterpret_cast<uint32_t *>(stage), *const tl = th + kMaxLines * kMaxLines;
+        static_assert(2 * 4 * kMaxLines * kMaxLines <= kStageBytes, "the table fits the epilogue's staging rows");
         const double wsc = SCALED ? ldexp(1.0, 15 - p.ew) : 1.0;  // |w| 2^(15 - ew) < 2^15: exact scaling
+        for (int e = tid; e < lines * lines; e += kThreads) {
+            const double wv = p.w[e] * wsc;
+            if constexpr (TF) {
+                const float h = to_tf32((float)wv);
+                th[e] = __float_as_uint(h);
+                if (SPLIT) tl[e] = __float_as_uint(to_tf32((float)(wv - (double)h)));
+            } else {
+                using O = Op<FORM == kBF16x3>;
+                const uint16_t h = O::bits(wv);
+                th[e] = h;
+                if (SPLIT) tl[e] = O::bits(wv - O::value(h));
+            }
+        }
+        __syncthreads();
         const int nelem = (31 + 2 * R) * nc * 8 * CE;
         for (int e = tid; e < nelem; e += kThreads) {
             const int j = e % CE, i = (e / CE) & 7, core = e / (8 * CE);
             const int d = core / nc - 15, idx = CE * (core % nc) + j + i - 7;
-            const double wv = (d >= 0 && d < lines && idx >= 0 && idx < lines) ? p.w[d * lines + idx] * wsc : 0.0;
+            const bool tap = d >= 0 && d < lines && idx >= 0 && idx < lines;
+            const uint32_t h = tap ? th[d * lines + idx] : 0u, l = SPLIT && tap ? tl[d * lines + idx] : 0u;
             if constexpr (TF) {
-                const float h = to_tf32((float)wv);
-                reinterpret_cast<float *>(Whi)[e] = h;
-                if (SPLIT) reinterpret_cast<float *>(Wlo)[e] = to_tf32((float)(wv - (double)h));
+                reinterpret_cast<uint32_t *>(Whi)[e] = h;
+                if (SPLIT) reinterpret_cast<uint32_t *>(Wlo)[e] = l;
             } else {
-                using O = Op<FORM == kBF16x3>;
-                const uint16_t h = O::bits(wv);
-                reinterpret_cast<uint16_t *>(Whi)[e] = h;
-                if (SPLIT) reinterpret_cast<uint16_t *>(Wlo)[e] = O::bits(wv - O::value(h));
+                reinterpret_cast<uint16_t *>(Whi)[e] = (uint16_t)h;
+                if (SPLIT) reinterpret_cast<uint16_t *>(Wlo)[e] = (uint16_t)l;
             }
         }
     }
