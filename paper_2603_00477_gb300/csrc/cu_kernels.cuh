@@ -723,7 +723,7 @@ constexpr int kMarchDepth = 8;  // ring rows per warp (a power of two)
 template <int SHAPE, int R, int T>
 __host__ __device__ constexpr bool march_has()
 {
-    return R <= 3 && (T == 1 || (T == 2 && (R == 1 || (SHAPE == 1 && R <= 3))));
+    return R <= 3 && (T == 1 || (T == 2 && (R <= 2 || SHAPE == 1)));
 }
 
 // Columns a warp yields.
@@ -748,9 +748,21 @@ __host__ __device__ constexpr int march_warp_floats()
     return 128 * (kMarchDepth + (VEC ? 0 : 1));
 }
 
+// Whether the products of column pairs run as packed FMAs (fma.rn.f32x2: the same
+// two roundings from one issue slot).  They take no constant-bank operand, so
+// they pay where the weights are in registers anyway (the batched kernel) or
+// where a weight is used often between loads: Box-2D2R at t = 2, 746 us a sweep
+// of 16384^2 where the tiled kernel took 1097.  In the other kernels here, which
+// read weights from the constant bank, they ran 0 to 10 % slower.
+template <int SHAPE, int R, int T>
+__host__ __device__ constexpr bool march_packs()
+{
+    return SHAPE == 0 && R == 2 && T == 2;
+}
+
 // One work item of a warp: output rows [y0, y1), the cw <= march_cols columns
 // from w0 + 4T on (w0: first column of the 128-column window, a multiple of 4 where VEC).
-template <int SHAPE, int R, int T, bool VEC, typename WT>
+template <int SHAPE, int R, int T, bool VEC, bool PACK, typename WT>
 __device__ __forceinline__ void march_strip(const float *__restrict__ in, float *__restrict__ out, const WT &wt,
                                             int64_t Ey, int64_t Ex, int64_t w0, int64_t y0, int64_t y1, int cw,
                                             float *ring)
@@ -793,11 +805,11 @@ __device__ __forceinline__ void march_strip(const float *__restrict__ in, float 
     cp_async_wait_group<0>();  // the previous item's rows have landed and are read
     __syncwarp();
     for (int i = 0; i < D - 1; ++i) load(i);
-    float acc[T][NS][4];
+    float2 acc[T][NS][2];
 #pragma unroll
     for (int s = 0; s < T; ++s)
 #pragma unroll
-        for (int m = 0; m < NS; ++m) acc[s][m][0] = acc[s][m][1] = acc[s][m][2] = acc[s][m][3] = 0.0f;
+        for (int m = 0; m < NS; ++m) acc[s][m][0] = acc[s][m][1] = make_float2(0.0f, 0.0f);
     // values of the rows R back, which the fixed boundary keeps (t > 1)
     float hist[T > 1 ? T - 1 : 1][NS][4];
     for (int base = 0; base < nrows; base += U) {
@@ -824,7 +836,7 @@ __device__ __forceinline__ void march_strip(const float *__restrict__ in, float 
                 float v[4 + 2 * R];
 #pragma unroll
                 for (int c = 0; c < R; ++c) {
-                    v[c] = __shfl_up_sync(0xffffffffu, q[4 - R + c], 1);
+                    v[c] = __shfl_up_sync(0xffffffffu, q[c + 4 - R], 1);
                     v[R + 4 + c] = __shfl_down_sync(0xffffffffu, q[c], 1);
                 }
 #pragma unroll
@@ -842,17 +854,24 @@ __device__ __forceinline__ void march_strip(const float *__restrict__ in, float 
                         const int k = tap_index<SHAPE, 2, R>(0, e - R, ox);
                         if (k >= 0) {
 #pragma unroll
-                            for (int c = 0; c < 4; ++c)
-                                acc[s][slot][c] = fmaf(wt.w[k], v[R + ox + c], acc[s][slot][c]);
+                            for (int c = 0; c < 2; ++c) {
+                                float2 &a = acc[s][slot][c];
+                                const float2 x = make_float2(v[R + ox + 2 * c], v[R + ox + 2 * c + 1]);
+                                if constexpr (PACK)
+                                    a = __ffma2_rn(make_float2(wt.w[k], wt.w[k]), x, a);
+                                else
+                                    a = make_float2(fmaf(wt.w[k], x.x, a.x), fmaf(wt.w[k], x.y, a.y));
+                            }
                         }
                     }
                 }
                 // output j - 2R is complete: slot (us + 1) mod NS
                 constexpr int done = (us + 1) % NS;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    q[c] = acc[s][done][c];
-                    acc[s][done][c] = 0.0f;
+                for (int c = 0; c < 2; ++c) {
+                    q[2 * c] = acc[s][done][c].x;
+                    q[2 * c + 1] = acc[s][done][c].y;
+                    acc[s][done][c] = make_float2(0.0f, 0.0f);
                 }
                 if constexpr (s < T - 1) {
                     // the halo keeps its value between the fused steps
@@ -905,7 +924,7 @@ __global__ void __launch_bounds__(kMarchThreads, (march_ctas<SHAPE, R, T>()))
     const int nwarps = (int)(gridDim.x * (kMarchThreads / 32));
     for (int item = (int)(blockIdx.x * (kMarchThreads / 32) + (threadIdx.x >> 5)); item < nitems; item += nwarps) {
         const int64_t y0 = R + (int64_t)(item / ncb) * seg;
-        march_strip<SHAPE, R, T, VEC>(in, out, wt, Ey, Ex, xb + (int64_t)(item % ncb) * CW - 4 * T, y0,
+        march_strip<SHAPE, R, T, VEC, march_packs<SHAPE, R, T>()>(in, out, wt, Ey, Ex, xb + (int64_t)(item % ncb) * CW - 4 * T, y0,
                                       min(y0 + seg, Ey - R), CW, ring);
     }
     cp_async_wait_group<0>();

@@ -77,7 +77,8 @@ __device__ __forceinline__ T ld_l2(const T *p)
 // down them on its own (cu::march_strip), so an item has no barrier inside.  The
 // shared-memory tiles below (the other depths and types) stage, wait and compute
 // in phases: a batch of 64 grids of 64 .. 4096 points a side, 20 steps, took 8.2 ms
-// with them and 3.4 ms here.
+// with them and 3.2 ms here (3.35 with scalar FMAs: the weights are in registers,
+// so the packed ones only save issue slots).
 template <int SHAPE, int R, int T, bool VEC>
 __device__ __noinline__ void march_tile(const GridDev &G, const float *__restrict__ wg, const float *src_g,
                                         float *dst_g, int tile, float *smem)
@@ -91,8 +92,8 @@ __device__ __noinline__ void march_tile(const GridDev &G, const float *__restric
     const int64_t c0 = (R - R % 4) + (int64_t)(tile % G.ntx) * G.bx + (int64_t)(warp % kcb) * G.mcw;
     const int64_t y1 = min(y0 + rows, G.ey - R);
     if (y0 < y1 && c0 < G.ex - R)
-        cu::march_strip<SHAPE, R, T, VEC>(src_g, dst_g, wt, G.ey, G.ex, c0 - 4 * T, y0, y1, G.mcw,
-                                          smem + warp * cu::march_warp_floats<VEC>());
+        cu::march_strip<SHAPE, R, T, VEC, true>(src_g, dst_g, wt, G.ey, G.ex, c0 - 4 * T, y0, y1, G.mcw,
+                                                smem + warp * cu::march_warp_floats<VEC>());
     cu::cp_async_wait_group<0>();
 }
 
@@ -364,7 +365,7 @@ bool march_has_host(int shape, int r, int t)
 {
     if (r < 1 || r > 3 || t < 1 || t > 2) return false;
     if (t == 1) return true;
-    return shape == STENCIL_BOX ? cu::march_has<0, 1, 2>() && r == 1
+    return shape == STENCIL_BOX ? (r == 1 && cu::march_has<0, 1, 2>()) || (r == 2 && cu::march_has<0, 2, 2>())
                                 : (r == 1 && cu::march_has<1, 1, 2>()) || (r == 2 && cu::march_has<1, 2, 2>()) ||
                                       (r == 3 && cu::march_has<1, 3, 2>());
 }
