@@ -90,6 +90,16 @@ __device__ __forceinline__ void cp_async_elem(void *smem_dst, const void *gmem_s
                  : "memory");
 }
 
+// Sweeps of a run follow each other on one stream, each reading what the last
+// wrote (launch_chained).  A sweep touches no global memory before the one in front
+// of it is complete and its writes are visible (chain_wait); it lets the next one's
+// blocks take their places (chain_next) as soon as its own have all started, or,
+// where a sweep is bound by the FMA pipes, when their work is done: blocks placed
+// earlier pile up on the SMs that finish first.  (FP64 Box-2D3R on 600 x 500, ten
+// sweeps: 296 us unchained, 403 us with chain_next at the start.)
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 
 template <int N>
@@ -513,6 +523,8 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
                const __grid_constant__ Weights<T, Taps<SHAPE, 2, R>::K> wt, int64_t Ey, int64_t Ex, int BY, int BX,
                int t, const Tiles tiles, int ntiles)
 {
+    if constexpr (sizeof(T) == 4) chain_next();
+    chain_wait();
     constexpr int KT = Taps<SHAPE, 2, R>::K;
     constexpr bool kSmemW = sizeof(T) == 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -690,6 +702,7 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
         cur ^= 1;
     }
     cp_async_wait_group<0>();
+    if constexpr (sizeof(T) == 8) chain_next();
 }
 
 // ---------------------------------------------------------------------------
@@ -918,6 +931,8 @@ __global__ void __launch_bounds__(kMarchThreads, (march_ctas<SHAPE, R, T>()))
                const __grid_constant__ Weights<float, Taps<SHAPE, 2, R>::K> wt, int64_t Ey, int64_t Ex, int ncb,
                int seg, int nitems, int xb)
 {
+    chain_next();
+    chain_wait();
     constexpr int CW = march_cols<R, T>();
     __shared__ __align__(16) float smem[(kMarchThreads / 32) * march_warp_floats<VEC>()];
     float *const ring = smem + (threadIdx.x >> 5) * march_warp_floats<VEC>();
@@ -939,6 +954,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                const __grid_constant__ Weights<T, Taps<SHAPE, 3, R>::K> wt, int64_t Ez, int64_t Ey, int64_t Ex,
                int BZ, int BY, int BX, int t, int tiles_x, int tiles_y, int ntiles)
 {
+    chain_wait();
     constexpr int KT = Taps<SHAPE, 3, R>::K;
     constexpr bool kSmemW = sizeof(T) == 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1049,6 +1065,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         cur ^= 1;
     }
     cp_async_wait_group<0>();
+    chain_next();
 }
 
 // ---------------------------------------------------------------------------
@@ -1168,6 +1185,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                 const __grid_constant__ Weights<T, Taps<SHAPE, 3, R>::K> wt, int64_t Ez, int64_t Ey, int64_t Ex,
                 int tiles_x, int tiles_y, int cz, int nitems)
 {
+    chain_wait();
     constexpr int KT = Taps<SHAPE, 3, R>::K;
     constexpr bool kSmemW = sizeof(T) == 8;
     constexpr int RPT = stream_rows_per_thread<T>(), BY = 16 * RPT, BX = 64;
@@ -1282,6 +1300,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
     }
     cp_async_wait_group<0>();
+    chain_next();
 }
 
 
@@ -1371,6 +1390,7 @@ __global__ void __launch_bounds__(kThreads, 2)
              const __grid_constant__ Weights<float, Taps<SHAPE, 3, R>::K> wt, int64_t Ez, int64_t Ey, int64_t Ex,
              int nq, int ns, int tiles_x, int tiles_y, int nitems, int cz, int xb)
 {
+    chain_wait();
     constexpr int TY = rot_rows_per_thread<SHAPE, R>(), NS = 2 * R + 1, NPL = kRotNPL;
     static_assert(R <= 3, "one quad of halo columns per side");
     extern __shared__ __align__(16) float ring[];
@@ -1549,6 +1569,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         cp_async_wait_group<0>();
     }
+    chain_next();
 }
 
 }  // namespace cu

@@ -53,10 +53,9 @@ stencil_status launch2d_march(const Plan &p, const void *in, void *out, cudaStre
     const int64_t per_cta = cu::kMarchThreads / 32;
     const unsigned grid =
         (unsigned)std::min<int64_t>((items + per_cta - 1) / per_cta, (int64_t)std::max(1, occ) * std::max(1, sms));
-    kern<<<grid, cu::kMarchThreads, 0, st>>>((const float *)in, (float *)out, wt, p.ext[1], p.ext[2], (int)ncb,
-                                             (int)seg, (int)items, xb);
-    note_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(kern, grid, cu::kMarchThreads, 0, st, (const float *)in,
+                                         (float *)out, wt, p.ext[1], p.ext[2], (int)ncb, (int)seg, (int)items, xb);
+    if (e == cudaSuccess) note_launch();
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu2d_march launch");
 }
 
@@ -110,10 +109,9 @@ stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStr
     if (ntiles > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const int64_t resident = (int64_t)std::max(1, occ_blocks) * std::max(1, sms);
     const unsigned grid = (unsigned)std::min<int64_t>(ntiles, resident);
-    kern<<<grid, cu::kThreads, smem, st>>>((const T *)in, (T *)out, wt, p.ext[1], p.ext[2], BY, BX, t, tiles,
-                                           (int)ntiles);
-    note_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(kern, grid, cu::kThreads, smem, st, (const T *)in, (T *)out, wt,
+                                         p.ext[1], p.ext[2], BY, BX, t, tiles, (int)ntiles);
+    if (e == cudaSuccess) note_launch();
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu2d_sweep launch");
 }
 
@@ -156,10 +154,9 @@ stencil_status launch3d_stream(const Plan &p, const void *in, void *out, cudaStr
     const int64_t items = (nz + cz - 1) / cz * tyy * txx;
     if (items > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const unsigned grid = (unsigned)std::min<int64_t>(items, (int64_t)std::max(1, occ) * std::max(1, sms));
-    kern<<<grid, cu::kThreads, smem, st>>>((const T *)in, (T *)out, wt, p.ext[0], p.ext[1], p.ext[2], (int)txx,
-                                           (int)tyy, (int)cz, (int)items);
-    note_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(kern, grid, cu::kThreads, smem, st, (const T *)in, (T *)out, wt,
+                                         p.ext[0], p.ext[1], p.ext[2], (int)txx, (int)tyy, (int)cz, (int)items);
+    if (e == cudaSuccess) note_launch();
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu3d_stream launch");
 }
 
@@ -201,10 +198,10 @@ stencil_status launch3d_rot(const Plan &p, const void *in, void *out, cudaStream
     const int64_t items = ((nz + cz - 1) / cz) * cols;
     if (items > 0x7fffffff || cz > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const unsigned grid = (unsigned)std::min<int64_t>(items, slots);
-    kern<<<grid, cu::kThreads, tile.smem, st>>>((const float *)in, (float *)out, wt, p.ext[0], p.ext[1], p.ext[2],
-                                                tile.nq, tile.ns, tile.tiles_x, tile.tiles_y, (int)items, (int)cz, xb);
-    note_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(kern, grid, cu::kThreads, tile.smem, st, (const float *)in,
+                                         (float *)out, wt, p.ext[0], p.ext[1], p.ext[2], tile.nq, tile.ns,
+                                         tile.tiles_x, tile.tiles_y, (int)items, (int)cz, xb);
+    if (e == cudaSuccess) note_launch();
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu3d_rot launch");
 }
 
@@ -245,10 +242,9 @@ stencil_status launch3d(const Plan &p, const void *in, void *out, int t, cudaStr
     if (ntiles > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const int64_t resident = (int64_t)std::max(1, occ_blocks) * std::max(1, sms);
     const unsigned grid = (unsigned)std::min<int64_t>(ntiles, resident);
-    kern<<<grid, cu::kThreads, smem, st>>>((const T *)in, (T *)out, wt, p.ext[0], p.ext[1], p.ext[2], BZ, BY, BX,
-                                           t, (int)tx, (int)ty, (int)ntiles);
-    note_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(kern, grid, cu::kThreads, smem, st, (const T *)in, (T *)out, wt,
+                                         p.ext[0], p.ext[1], p.ext[2], BZ, BY, BX, t, (int)tx, (int)ty, (int)ntiles);
+    if (e == cudaSuccess) note_launch();
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu3d_sweep launch");
 }
 

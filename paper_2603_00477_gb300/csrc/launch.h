@@ -69,6 +69,34 @@ stencil_status ensure_smem(const void *func, size_t bytes);
 // cached for the process (thread safe).
 stencil_status occupancy(const void *func, int threads, size_t smem, int *blocks);
 
+// Launch a sweep kernel that begins with cu::chain_wait() behind the kernel
+// that writes its input: its blocks may be placed while that kernel's last ones
+// run (programmatic stream serialisation), which takes the gap between dependent
+// launches out of a run of short sweeps.  The attribute also holds under stream
+// capture.  The kernel in front must be a kernel of the same run (the halo copy or
+// a sweep).
+// Measured, unchained before: Star-2D1R FP64 512^2, 10 steps 86 -> 56 us;
+// Star-2D2R FP32 1021 x 1531, 20 steps 107 -> 87 us; Box-2D3R FP64 230 x 310,
+// 10 steps 127 -> 103 us; Star-3D1R FP32 64 x 65 x 66, 6 steps 41 -> 31 us;
+// long sweeps 0 to 1.5 %.
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+                           A &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    return e == cudaSuccess ? cudaGetLastError() : (cudaGetLastError(), e);
+}
+
 stencil_status cuda_fail(cudaError_t e, const char *what);
 
 }  // namespace gbs
