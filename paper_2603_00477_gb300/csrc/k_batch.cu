@@ -584,8 +584,8 @@ stencil_status check_run_args(stencil_batch *b, const void *const *ins, void *co
 // batch leaves warps idle: a sweep of a grid then takes as long as one item, 2 t r
 // rows and a start-up longer than its rows.  Nine grids of 64 .. 512 a side, 14
 // steps: 336 us with the rule by grid alone (221 with staged tiles), 215 us with it;
-// 32 grids of 64 .. 1024, 18 steps: 559 -> 490 us.  Otherwise one staging + one work buffer per work item, the CUDA-core
-// default tile halved until the grown tile pair fits the per-item budget.
+// 32 grids of 64 .. 1024, 18 steps: 559 -> 490 us.  Otherwise one staging + one
+// work buffer per work item, the CUDA-core default tile halved until the grown tile pair fits the per-item budget.
 void batch_tile(Plan *p, int64_t points)
 {
     int tile[3];
