@@ -1399,7 +1399,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int PH = ns * TY + 2 * R, PQ = nq + 2, PW = 4 * PQ, quads = PH * PQ, PE = 4 * quads;
     float *const turn = ring + (size_t)NPL * PE + (tid >> 5) * 128;  // word rows: a warp's 32 quads
     const int64_t nz = Ez - 2 * R, ny = Ey - 2 * R, nx = Ex - 2 * R, plane = Ey * Ex;
-    const int ex32 = (int)Ex;  // a stored row holds < 2^31 values, and a stored plane too
+    const int ex32 = (int)Ex;  // a stored plane holds < 2^31 values (rot3d_plane_fits)
 
     for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
         const int bx = item % tiles_x, by = (item / tiles_x) % tiles_y, bz = item / (tiles_x * tiles_y);

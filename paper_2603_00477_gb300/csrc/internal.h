@@ -104,6 +104,11 @@ const std::vector<double> &composite(const Plan &p, int t);
 
 stencil_status dispatch(Plan *p);  // fills path/precision/t/tile/info
 
+// Whether the 3-D marching kernel (cu3d_rot) can run a grid with stored planes of
+// ey x ex values: its copies and stores hold the offset inside a plane in 32 bits.
+// Larger planes (8.6 GB and up) take the streaming kernel, whose offsets are 64 bits wide.
+inline bool rot3d_plane_fits(int64_t ey, int64_t ex) { return ey * ex <= INT32_MAX; }
+
 // kernel-family availability (host knowledge of what the .cu files build)
 bool cu_supported(int shape, int d, int r);
 void cu_default_tile(const Plan &p, int t, int tile[3]);

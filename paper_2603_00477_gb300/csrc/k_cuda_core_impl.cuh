@@ -209,12 +209,13 @@ template <typename T, int SHAPE, int R>
 stencil_status launch3d(const Plan &p, const void *in, void *out, int t, cudaStream_t st)
 {
     if (t == 1) {
-        // FP32 star r <= 3 and box r = 1: rotating partial sums; the rest streams
+        // FP32 star r <= 3 and box r = 1 with planes of 32-bit offsets: rotating partial sums; the rest streams
         if constexpr (sizeof(T) == 4 && ((SHAPE == 1 && R <= 3) || (SHAPE == 0 && R == 1)))
-            return p.ext[2] % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0 &&
-                           reinterpret_cast<uintptr_t>(out) % 16 == 0
-                       ? launch3d_rot<SHAPE, R, true>(p, in, out, st)
-                       : launch3d_rot<SHAPE, R, false>(p, in, out, st);
+            if (rot3d_plane_fits(p.ext[1], p.ext[2]))
+                return p.ext[2] % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0 &&
+                               reinterpret_cast<uintptr_t>(out) % 16 == 0
+                           ? launch3d_rot<SHAPE, R, true>(p, in, out, st)
+                           : launch3d_rot<SHAPE, R, false>(p, in, out, st);
         return launch3d_stream<T, SHAPE, R>(p, in, out, st);
     }
     using Wt = cu::Weights<T, cu::Taps<SHAPE, 3, R>::K>;
