@@ -34,12 +34,18 @@
 // bit), the plane distance (TF32) or one row (the odd chunk).  No im2col copy.
 //
 // The 16-bit forms scale each tile by a power of two (FP16 has 5 exponent
-// bits) and the weights likewise; the epilogue undoes both exactly.  A tile is
-// read once: it is converted with the scale of the CTA's previous tile while
-// its largest |x| is found, and converted again only if that scale would
-// overflow or leave the largest value below 2^7 (the FP16 normal range starts
-// at 2^-14, so values down to 2^-21 of the tile's largest keep 11 bits, and the
-// lo parts of f16x3 stay exact to 2^-31 of it).  TF32 needs no scale.
+// bits) and the weights likewise; the epilogue undoes both exactly.  The tile's
+// largest |x| lands in [2^14, 65504]: the FP16 normal range starts at 2^-14, so
+// values down to 2^-28 of the largest keep 11 bits, and the lo parts of f16x3
+// stay exact to 2^-38 of it.  A tile is read once where that can be had: the
+// epilogue warps, which wait most of the time, look at 512 values spread over the
+// tile two tiles ahead, and the scale that puts the largest of those in
+// [2^14, 2^15) cannot be below the rule's, so a tile converted with it keeps at
+// least those bits; it is converted again, from L2, only if a value outside the
+// sample is 2 to 4 times larger than all of it and would overflow.  The scale
+// depends on the tile alone.  (The scale of the CTA's tile before, kept as long as
+// the largest value fell in [2^7, 2^15), took seven bits off the small values
+// beside a large one.)  TF32 needs no scale.
 //
 // A tile is hx = 1 or 2 such column groups of 64 side by side: an MMA of N = 128
 // takes exactly half the time of one of N = 256 (64 / 128 cycles; ~50 is the
@@ -62,7 +68,7 @@
 // Measured, one fused sweep (line form before, block form now): Box-2D2R f16
 // t = 4 on 16384^2 776 -> 476 us (HBM floor 317; a plain tiled copy that
 // re-reads the same halo 415), f16x3 t = 4 on 7001 x 6007 (unaligned rows)
-// 433 -> 171 us, Box-2D1R TF32 t = 7 on 10240^2 654 (2:4 sparse form) -> 265 us.
+// 433 -> 178 us (171 without the sample), Box-2D1R TF32 t = 7 on 10240^2 654 (2:4 sparse form) -> 265 us.
 // The loaders set the pace (15k cycles per 256 x 128 tile; MMAs 6.2k).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -166,12 +172,23 @@ struct Op<true> {
     }
 };
 
+// The scale exponent that puts a largest |x| of these bits in [2^14, 2^15) (clamped to FP32's range).
+__device__ __forceinline__ int scale_of(unsigned mx)
+{
+    return max(-126, min(127, 141 - (int)(mx >> 23)));  // |x| < 2^((mx >> 23) - 126)
+}
+
 // Largest |x| seen so far, as an unsigned integer (IEEE order).
 __device__ __forceinline__ unsigned max_abs(unsigned m, const float4 &v)
 {
     return max(m, max(max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu),
                       max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu)));
 }
+
+// The largest scaled |x| a tile may be converted with: FP16's largest number; BF16 has FP32's range, and its
+// sums of 625 products with weights below 2^15 stay in FP32's range from 2^64 too.
+template <int FORM>
+constexpr float kMaxOperand = FORM == kBF16x3 ? 0x1p64f : 65504.0f;
 
 // Convert the four columns of item i (row i / (2 pc), columns 4 (i mod 2 pc) ..)
 // and store them to the operand buffer: 8 bytes (16-bit forms) or one 16-byte
@@ -220,8 +237,10 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
     uint64_t *accfree = reinterpret_cast<uint64_t *>(smem + 48);  // [2] accumulator drained
     uint64_t *maxb = reinterpret_cast<uint64_t *>(smem + 64);     // [2] exponent exchange
     uint64_t *eub = reinterpret_cast<uint64_t *>(smem + 80);      // [4] a tile's scale published
-    int *wmax = reinterpret_cast<int *>(smem + 128);              // [2][kLoadWarps]
-    int *eus = reinterpret_cast<int *>(smem + 256);               // [4] input scale exponent per tile
+    uint64_t *smpb = reinterpret_cast<uint64_t *>(smem + 112);    // [4] a tile's sample taken
+    unsigned *wmax = reinterpret_cast<unsigned *>(smem + 160);    // [2][kLoadWarps] largest |x| of a tile
+    unsigned *wsmp = reinterpret_cast<unsigned *>(smem + 288);    // [4][kEpiWarps] and of its sample
+    int *eus = reinterpret_cast<int *>(smem + 416);               // [4] input scale exponent per tile
     const int R = p.R, lines = 2 * R + 1, nc = p.nc, pc = p.pc, gn = p.gn, hx = p.hx, nbuf = p.nbuf;
     const uint32_t strip_bytes = (uint32_t)(31 + 2 * R) * nc * 128;
     const uint32_t in_bytes = p.in_bytes;
@@ -250,7 +269,10 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
             mbar_init(&accfree[b], 32 * kEpiWarps);
             mbar_init(&maxb[b], kLoaders);
         }
-        for (int s = 0; s < 4; ++s) mbar_init(&eub[s], 1);
+        for (int s = 0; s < 4; ++s) {
+            mbar_init(&eub[s], 1);
+            mbar_init(&smpb[s], kEpiWarps);
+        }
         fence_mbar_init();
     }
     // Weight strip: core matrix (L, c), L = ky + g, holds line L - 15.  Each
@@ -442,7 +464,6 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
             }
         };
         bool started = false;  // v holds this tile's first items
-        int es = 12;  // the scale the next tile is first tried with: the previous tile's
         int k = 0;
         for (int id = blockIdx.x; id < ntiles; id += gridDim.x, ++k) {
             const int b = k & 1;
@@ -452,6 +473,14 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
             if (nbuf == 2 && k >= 2 && !bounded_wait(&done[b], ((k - 2) >> 1) & 1, kWaitCycles)) break;
             if (nbuf == 1 && k >= 1 && !bounded_wait(&done[b ^ 1], ((k - 1) >> 1) & 1, kWaitCycles)) break;
             unsigned char *hi = ibase + (nbuf == 2 ? b : 0) * in_bytes, *lo = hi + nbuf * in_bytes;
+            int es = 0;  // the tile's scale exponent: first the sample's
+            if constexpr (SCALED) {
+                if (!bounded_wait(&smpb[k & 3], (k >> 2) & 1, kWaitCycles)) break;
+                unsigned m = 0;
+#pragma unroll
+                for (int w = 0; w < kEpiWarps; ++w) m = max(m, wsmp[(k & 3) * kEpiWarps + w]);
+                es = scale_of(m);
+            }
             // Interior tiles: no per-load bounds tests.  Rows that are not 16-byte
             // multiples are read as the two aligned 16-byte words around each
             // quad (the region then keeps a stored row free above and below, so
@@ -538,21 +567,20 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
                     }
                 }
                 if (!SCALED || attempt == 1) break;
-                const int mx = (int)(__reduce_max_sync(0xffffffffu, mxu) >> 23);
-                if (lane == 0) wmax[b * kLoadWarps + warp] = mx;
+                mxu = __reduce_max_sync(0xffffffffu, mxu);
+                if (lane == 0) wmax[b * kLoadWarps + warp] = mxu;
                 __syncwarp();
                 mbar_arrive(&maxb[b]);
                 if (!bounded_wait(&maxb[b], (k >> 1) & 1, kWaitCycles)) {
                     break;  // the abort flag is set
                 }
-                int emax = wmax[b * kLoadWarps];
+                mxu = wmax[b * kLoadWarps];
 #pragma unroll
-                for (int w = 1; w < kLoadWarps; ++w) emax = max(emax, wmax[b * kLoadWarps + w]);
-                // |x| < 2^(emax - 126): keep the scale while 2^7 <= max |x| 2^es < 2^15 or the tile is
-                // zero, else convert again with the largest value in [2^11, 2^12)
-                const int top = emax - 126 + es;
-                if (emax == 0 || (top <= 15 && top >= 8)) break;
-                es = max(-126, min(127, 138 - emax));
+                for (int w = 1; w < kLoadWarps; ++w) mxu = max(mxu, wmax[b * kLoadWarps + w]);
+                // keep the scale if it is the rule's for the whole tile or the largest value still fits
+                const int want = scale_of(mxu);
+                if (es == want || __uint_as_float(mxu) * pow2f(es) <= kMaxOperand<FORM>) break;
+                es = want;
                 started = false;  // converting again reloads the tile into v
             }
             if (*(volatile int *)abort_flag) break;
@@ -575,12 +603,50 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
         const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16);
         float *st = stage + (warp - kEpiWarp) * 4 * kStageRow;
         float *put_at = st + (3 - (lane >> 3)) * kStageRow + 7 - (lane & 7);
+        // This thread's two of the 512 values of a sample of tile id: 8 values of a row at 64 places spread over
+        // the staged region (0 outside the stored array).  Whole 32-byte sectors, because the tile itself comes
+        // three tiles later and HBM may read them twice: single values cost f16 on 16384^2 10 %.
+        auto take_sample = [&](int id, float *x) {
+            x[0] = x[1] = 0.0f;
+            if (id >= ntiles) return;
+            const int rows = kBY * gn + 2 * R, place = (tid - 32 * kEpiWarp) >> 2;
+            int64_t Y0, X0;
+            origin(id, &Y0, &X0);
+            const int64_t gy = Y0 - R + place * rows / 64;
+            const int64_t gx = X0 - R + (37 * place & 63) * (8 * pc - 8) / 63 + 2 * (lane & 3);
+            if (gy < 0 || gy >= Ey) return;
+            const float *s = in + gy * Ex + gx;
+            if (gx >= 0 && gx < Ex) x[0] = __ldcg(s);
+            if (gx + 1 >= 0 && gx + 1 < Ex) x[1] = __ldcg(s + 1);
+        };
+        // post the largest of a sample as that of the CTA's tile k (slot k & 3 was last read for tile k - 4, which
+        // the loaders left before the epilogue of tile k - 3 could end)
+        auto post_sample = [&](int k, const float *x) {
+            const unsigned m = __reduce_max_sync(
+                0xffffffffu, max(__float_as_uint(x[0]) & 0x7fffffffu, __float_as_uint(x[1]) & 0x7fffffffu));
+            if (lane == 0) {
+                wsmp[(k & 3) * kEpiWarps + warp - kEpiWarp] = m;
+                mbar_arrive(&smpb[k & 3]);
+            }
+            __syncwarp();
+        };
+        float ahead[2];  // the sample of the tile two ahead, in flight while a tile is written
         int k = 0;
         bool ok = true;
+        if constexpr (SCALED) {
+            float next[2];
+            take_sample(blockIdx.x, ahead);
+            take_sample(blockIdx.x + gridDim.x, next);
+            post_sample(0, ahead);
+            post_sample(1, next);
+            take_sample(blockIdx.x + 2 * gridDim.x, ahead);
+        }
         for (int id = blockIdx.x; id < ntiles; id += gridDim.x, ++k) {
             const int b = k & 1;
             int es = 0;
             if constexpr (SCALED) {
+                post_sample(k + 2, ahead);
+                take_sample(id + 3 * (int)gridDim.x, ahead);
                 if (!bounded_wait(&eub[k & 3], (k >> 2) & 1, kWaitCycles)) {
                     ok = false;
                     break;
