@@ -141,12 +141,12 @@ __device__ __forceinline__ void march_item(const GridDev &G, const float *wg, co
     else march_tile<SHAPE, R, 1, false>(G, wg, src, dst, tile, smem);
 }
 
-// One item: tile `tile` of grid G, sweep s (depth t_s) from src to dst.
-template <typename T, int SHAPE, int R, int V>
+// One item: tile `tile` of grid G, sweep s (depth t_s) from src to dst.  MARCH: the kernel has the marching path.
+template <typename T, int SHAPE, int R, int V, bool MARCH>
 __device__ void run_item(const GridDev &G, const T *__restrict__ wg, const T *src_g, T *dst_g, int tile, int s,
                          int ts, unsigned char *smem)
 {
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (MARCH) {
         if (G.mcw > 0) {
             march_item<SHAPE, R>(G, wg, src_g, dst_g, tile, s, ts, reinterpret_cast<float *>(smem));
             return;
@@ -267,10 +267,10 @@ __device__ void run_item(const GridDev &G, const T *__restrict__ wg, const T *sr
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1)
-    batch_sweeps(const GridDev *__restrict__ grids, const Item *__restrict__ items, int nitems,
-                 const T *__restrict__ wtab, int *done, Ctl *ctl, unsigned long long wait_cycles, int block_sweep)
+template <typename T, bool MARCH>
+__device__ __forceinline__ void sweep_items(const GridDev *__restrict__ grids, const Item *__restrict__ items,
+                                            int nitems, const T *__restrict__ wtab, int *done, Ctl *ctl,
+                                            unsigned long long wait_cycles, int block_sweep)
 {
     constexpr int V = sizeof(T) == 8 ? 4 : 8;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -304,18 +304,40 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1)
         T *dst = reinterpret_cast<T *>(((G.nsweeps - 1 - it.s) % 2 == 0) ? G.out : G.pp);
         const T *wg = wtab + G.woff;
         switch (G.kind) {
-        case 0 * 4 + 1: run_item<T, 0, 1, V>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
-        case 0 * 4 + 2: run_item<T, 0, 2, V>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
-        case 0 * 4 + 3: run_item<T, 0, 3, V>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
-        case 1 * 4 + 1: run_item<T, 1, 1, V>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
-        case 1 * 4 + 2: run_item<T, 1, 2, V>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
-        case 1 * 4 + 3: run_item<T, 1, 3, V>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
+        case 0 * 4 + 1: run_item<T, 0, 1, V, MARCH>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
+        case 0 * 4 + 2: run_item<T, 0, 2, V, MARCH>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
+        case 0 * 4 + 3: run_item<T, 0, 3, V, MARCH>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
+        case 1 * 4 + 1: run_item<T, 1, 1, V, MARCH>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
+        case 1 * 4 + 2: run_item<T, 1, 2, V, MARCH>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
+        case 1 * 4 + 3: run_item<T, 1, 3, V, MARCH>(G, wg, src, dst, it.tile, it.s, ts, smem); break;
         default: break;
         }
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) atomicAdd(done + G.doff + it.s, 1);
     }
+}
+
+// Shared-memory tiles only: every FP64 batch, and FP32 batches without marching
+// grids.  80 registers in FP32, three CTAs per SM.
+template <typename T>
+__global__ void __launch_bounds__(kThreads)
+    batch_sweeps(const GridDev *__restrict__ grids, const Item *__restrict__ items, int nitems,
+                 const T *__restrict__ wtab, int *done, Ctl *ctl, unsigned long long wait_cycles, int block_sweep)
+{
+    sweep_items<T, false>(grids, items, nitems, wtab, done, ctl, wait_cycles, block_sweep);
+}
+
+// FP32 batches with marching grids.  The marching path keeps weights and partial sums
+// in registers (128, two CTAs per SM); shared-memory tiles run here at 1.6 to 1.8
+// times the time they take above (30 grids of 500 x 500, t = 3 and 4), which is why the
+// two are separate kernels and march_pays counts the tiles.
+__global__ void __launch_bounds__(kThreads, 2)
+    batch_sweeps_march(const GridDev *__restrict__ grids, const Item *__restrict__ items, int nitems,
+                       const float *__restrict__ wtab, int *done, Ctl *ctl, unsigned long long wait_cycles,
+                       int block_sweep)
+{
+    sweep_items<float, true>(grids, items, nitems, wtab, done, ctl, wait_cycles, block_sweep);
 }
 
 }  // namespace bt
@@ -354,6 +376,7 @@ struct stencil_batch {
     unsigned long long wait_cycles = gbs::bt::kWaitCycles;  // bounded dependency wait
     int block_sweep = -1;  // test hook: sweep whose items wait on a counter nothing increments
     int precision = STENCIL_PREC_NATIVE;  // forms the autotuner may use for FP32 grids
+    bool march_kernel = false;  // run batch_sweeps_march without marching grids too (the autotuner's measurements)
     gbs::BatchCache cache;
 };
 
@@ -478,14 +501,18 @@ stencil_status launch_batch(stencil_batch *b, const Layout &L, const void *const
     if (L.nitems == 0) return launch_tc_grids(b, L, ins, outs, steps, st);
     size_t smem = 0;
     const size_t es = b->dtype == STENCIL_F64 ? 8 : 4;
+    bool march = b->march_kernel;
     for (auto &g : b->grids) {
         if (!g.on_cu()) continue;
         const int R = g.plan.pat.r, t = g.plan.t;
-        smem = std::max(smem, march_columns(g.plan)
-                                  ? (size_t)(bt::kThreads / 32) * cu::march_warp_floats<false>() * sizeof(float)
-                                  : batch_item_smem(g.plan.tile[1], g.plan.tile[2], t, R, es));
+        const bool m = march_columns(g.plan) > 0;
+        march = march || m;
+        smem = std::max(smem, m ? (size_t)(bt::kThreads / 32) * cu::march_warp_floats<false>() * sizeof(float)
+                                : batch_item_smem(g.plan.tile[1], g.plan.tile[2], t, R, es));
     }
-    const void *fn = b->dtype == STENCIL_F64 ? (const void *)bt::batch_sweeps<double> : (const void *)bt::batch_sweeps<float>;
+    const void *fn = b->dtype == STENCIL_F64 ? (const void *)bt::batch_sweeps<double>
+                     : march                 ? (const void *)bt::batch_sweeps_march
+                                             : (const void *)bt::batch_sweeps<float>;
     stencil_status s = ensure_smem(fn, smem);
     if (s != STENCIL_OK) return s;
     int occ = 0, dev = 0, sms = 0;
@@ -501,6 +528,9 @@ stencil_status launch_batch(stencil_batch *b, const Layout &L, const void *const
     if (b->dtype == STENCIL_F64)
         bt::batch_sweeps<double><<<grid, bt::kThreads, smem, st>>>(gd, items, L.nitems, (const double *)(ws + L.w_off),
                                                                    done, ctl, b->wait_cycles, b->block_sweep);
+    else if (march)
+        bt::batch_sweeps_march<<<grid, bt::kThreads, smem, st>>>(gd, items, L.nitems, (const float *)(ws + L.w_off),
+                                                                 done, ctl, b->wait_cycles, b->block_sweep);
     else
         bt::batch_sweeps<float><<<grid, bt::kThreads, smem, st>>>(gd, items, L.nitems, (const float *)(ws + L.w_off),
                                                                   done, ctl, b->wait_cycles, b->block_sweep);
@@ -578,37 +608,89 @@ stencil_status check_run_args(stencil_batch *b, const void *const *ins, void *co
     return STENCIL_OK;
 }
 
-// The default tile of a grid in a batch of `points` interior points.  Marching
-// path: two strips of columns (one on narrow grids) and 32 rows per warp, fewer
-// on small grids so that they have tiles enough, and fewer still where the whole
-// batch leaves warps idle: a sweep of a grid then takes as long as one item, 2 t r
-// rows and a start-up longer than its rows.  Nine grids of 64 .. 512 a side, 14
-// steps: 336 us with the rule by grid alone (221 with staged tiles), 215 us with it;
-// 32 grids of 64 .. 1024, 18 steps: 559 -> 490 us.  Otherwise one staging + one
-// work buffer per work item, the CUDA-core default tile halved until the grown tile pair fits the per-item budget.
-void batch_tile(Plan *p, int64_t points)
+bool march_capable(const Plan &p)
+{
+    return p.dtype == STENCIL_F32 && march_has_host(p.pat.shape, p.pat.r, p.t);
+}
+
+// Marching tile: two strips of columns (one on narrow grids) and at most `rows` rows per warp, fewer on small grids.
+void march_grid_tile(Plan *p, int rows)
+{
+    const int cw = 4 * (32 - 2 * p->t), kcb = p->dims[2] + p->pat.r % 4 > cw ? 2 : 1;
+    rows = std::min(rows, p->n_interior >= (1 << 20) ? 32 : (p->n_interior >= (1 << 16) ? 16 : 8));
+    p->tile[0] = p->info.tile[0] = 1;
+    p->tile[1] = p->info.tile[1] = rows * (8 / kcb);
+    p->tile[2] = p->info.tile[2] = cw * kcb;
+}
+
+// Shared-memory tile: one staging + one work buffer per work item, the CUDA-core default tile halved until the
+// grown tile pair fits the per-item budget.
+void staged_grid_tile(Plan *p)
 {
     int tile[3];
-    if (p->dtype == STENCIL_F32 && march_has_host(p->pat.shape, p->pat.r, p->t)) {
-        const int cw = 4 * (32 - 2 * p->t), kcb = p->dims[2] + p->pat.r % 4 > cw ? 2 : 1;
-        const int64_t warps = (int64_t)kBatchSms * 2 * (bt::kThreads / 32), share = points / (warps * cw);
-        int rows = p->n_interior >= (1 << 20) ? 32 : (p->n_interior >= (1 << 16) ? 16 : 8);
-        while (rows > 4 && share < rows) rows /= 2;
-        p->tile[0] = p->info.tile[0] = 1;
-        p->tile[1] = p->info.tile[1] = rows * (8 / kcb);
-        p->tile[2] = p->info.tile[2] = cw * kcb;
-        return;
-    }
     cu_default_tile(*p, p->t, tile);
     for (;;) {
         const size_t bytes = batch_item_smem(tile[1], tile[2], p->t, p->pat.r, p->elem_bytes());
         if (bytes <= kBatchItemSmem || (tile[1] <= 16 && tile[2] <= 16)) break;
         if (tile[2] >= tile[1]) tile[2] /= 2; else tile[1] /= 2;
     }
-    for (int k = 0; k < 3; k++) p->tile[k] = tile[k];
-    p->info.tile[0] = tile[0];
-    p->info.tile[1] = tile[1];
-    p->info.tile[2] = tile[2];
+    for (int k = 0; k < 3; k++) p->tile[k] = p->info.tile[k] = tile[k];
+}
+
+// Whether the grids `cu` of a batch take the marching path where they have it.
+// Measured, marching kernel against staged tiles only, 8 steps:
+//  * mixed batches: the marching kernel runs staged tiles at two CTAs per SM instead
+//    of three.  Ten grids of 300 a side, Star-2D2R beside Box-2D3R at t = 2 (staged):
+//    40 % of them staged 0.95, 50 % 1.06, 70 % 1.26 of the time.
+//  * small batches, where the marching kernel's few long items leave the chip idle.
+//    K t is a measure of an item's length.  16 grids of 64 (122,000 points): Box-2D3R
+//    (49) 1.26, Box-2D2R t = 2 (50) 1.28, Star-2D3R t = 2 (26) 1.15, Box-2D2R (25) 1.07,
+//    Star-2D2R t = 2 (18) 1.04, Star-2D1R t = 2 (10) 0.91; 4 of 64 (26,000): 1.09, 1.05, 1.05,
+//    0.91, 0.89, 0.81; 16 of 100 (244,000): 1.02, 1.01, 0.91, 0.86, 0.86, 0.76.
+//  * Box-2D3R alone, whose sweeps do not overlap another grid's: 500 x 500
+//    0.85, 800 x 800 1.01, 1200 x 1200 1.16 (1.48 with items of two rounds), 2500 x 2500 1.06.
+bool march_pays(const std::vector<Plan *> &cu)
+{
+    int64_t points = 0, in_tiles = 0;
+    int heaviest = 0;
+    for (const Plan *p : cu) {
+        points += p->n_interior;
+        if (!march_capable(*p)) in_tiles += p->n_interior;
+        else heaviest = std::max(heaviest, p->pat.K * p->t);
+    }
+    if (in_tiles > 0.45 * points) return false;
+    if (cu.size() == 1 && cu[0]->pat.K >= 40 && points < 8000000) return false;
+    const int64_t small = 220000, smaller = 100000;
+    return !(points < small && heaviest >= (points < smaller ? 40 : 18));
+}
+
+// The default tiles of a batch's grids on CUDA cores.
+void batch_tiles(const std::vector<Plan *> &cu)
+{
+    if (!march_pays(cu)) {
+        for (Plan *p : cu) staged_grid_tile(p);
+        return;
+    }
+    // Rows per warp: fewer where the whole batch leaves warps idle, because a sweep of a grid then takes as long as
+    // one item, 2 t r rows and a start-up longer than its rows.  Nine grids of 64 .. 512 a side, 14 steps: 336 us with
+    // 8 rows (221 staged), 215 us with 4; 32 grids of 64 .. 1024, 18 steps: 559 -> 490 us.
+    int64_t points = 0;
+    for (const Plan *p : cu) points += p->n_interior;
+    const int64_t warps = (int64_t)kBatchSms * 2 * (bt::kThreads / 32);
+    for (Plan *p : cu) {
+        if (!march_capable(*p)) {
+            staged_grid_tile(p);
+            continue;
+        }
+        const int64_t share = points / (warps * 4 * (32 - 2 * p->t));
+        int rows = 32;
+        while (rows > 4 && share < rows) rows /= 2;
+        march_grid_tile(p, rows);
+        // a grid alone: its items also fill whole rounds of the resident CTAs badly (1200 x 1200, Box-2D2R: 375 items
+        // of 4 rows are two rounds, 190 of 8 one)
+        if (cu.size() == 1 && rows < 32 && ntiles_of(*p) > 2 * kBatchSms && ntiles_of(*p) < 4 * kBatchSms)
+            march_grid_tile(p, 2 * rows);
+    }
 }
 
 void drop_graph(BatchCache &c)
@@ -660,9 +742,9 @@ try {
         stencil_plan_destroy(p);
         b->grids.push_back(std::move(g));
     }
-    int64_t points = 0;
-    for (auto &g : b->grids) points += g.plan.n_interior;
-    for (auto &g : b->grids) batch_tile(&g.plan, points);
+    std::vector<Plan *> cu;
+    for (auto &g : b->grids) cu.push_back(&g.plan);
+    batch_tiles(cu);
     *batch = b;
     return STENCIL_OK;
 } catch (...) {
@@ -823,8 +905,6 @@ try {
         else if (vs == "sparse_tensor_core") path = STENCIL_PATH_SPARSE_TENSOR_CORE;
         else return fail(STENCIL_ERR_INVALID_ARG, "batch path must be auto|cuda_core|tensor_core|sparse_tensor_core");
         std::vector<Plan> plans;
-        int64_t points = 0;
-        for (auto &g : batch->grids) points += g.plan.n_interior;
         for (auto &g : batch->grids) {
             Plan q = g.plan;
             q.req_path = path;
@@ -832,9 +912,12 @@ try {
             q.req_tile[0] = q.req_tile[1] = q.req_tile[2] = 0;
             stencil_status s = dispatch(&q);
             if (s != STENCIL_OK) return s;
-            if (q.path == STENCIL_PATH_CUDA_CORE) batch_tile(&q, points);
             plans.push_back(q);
         }
+        std::vector<Plan *> cu;
+        for (auto &q : plans)
+            if (q.path == STENCIL_PATH_CUDA_CORE) cu.push_back(&q);
+        batch_tiles(cu);
         for (size_t i = 0; i < plans.size(); i++) batch->grids[i].plan = plans[i];
         drop_graph(batch->cache);
         return STENCIL_OK;
@@ -905,6 +988,9 @@ try {
         int path, prec, t, ty, tx;
         double model, measured;
     };
+    // a class is measured alone, in the kernel that it will share with the others
+    bool march_kernel = false;
+    for (auto &g : batch->grids) march_kernel = march_kernel || (g.on_cu() && march_columns(g.plan) > 0);
     int nres = 0, cls = 0;
     for (auto &kv : classes) {
         const std::vector<int> &members = kv.second;
@@ -989,6 +1075,7 @@ try {
             sub.ws = batch->ws;
             sub.ws_bytes = batch->ws_bytes;
             sub.wait_cycles = batch->wait_cycles;
+            sub.march_kernel = march_kernel && c.path == STENCIL_PATH_CUDA_CORE;
             std::vector<const void *> sin;
             std::vector<void *> sout;
             bool ok = true;
