@@ -8,6 +8,7 @@
 
 #include "cu_kernels.cuh"
 #include "launch.h"
+#include "launch_rules.h"
 
 namespace gbs {
 namespace cuimpl {
@@ -136,21 +137,7 @@ stencil_status launch3d_stream(const Plan &p, const void *in, void *out, cudaStr
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int BY = 16 * cu::stream_rows_per_thread<T>(), BX = 64;
     const int64_t tyy = (p.dims[1] + BY - 1) / BY, txx = (p.dims[2] + BX - 1) / BX, nz = p.dims[0];
-    // Planes per chunk: an SM's CTAs share its FMA pipe, so the time is about
-    // (items of the busiest SM) x (planes + a start-up worth one plane).  With
-    // 64 planes a 256^3 grid was 256 items on 152 SMs, two on most and one on
-    // the rest (84 %); 37 planes give
-    // each SM 2.9 items: Box-3D1R FP64 908 -> 778 us per sweep
-    const int64_t nsm = std::max(1, sms);
-    int64_t cz = nz, cost = -1;
-    for (int64_t n = 1; n <= std::min<int64_t>(nz, 64); n++) {
-        const int64_t c = (nz + n - 1) / n, it = (nz + c - 1) / c * tyy * txx;
-        const int64_t v = (it + nsm - 1) / nsm * (c + 1);
-        if (cost < 0 || v < cost) {
-            cost = v;
-            cz = c;
-        }
-    }
+    const int64_t cz = stream_planes(nz, tyy * txx, std::max(1, occ), std::max(1, sms));
     const int64_t items = (nz + cz - 1) / cz * tyy * txx;
     if (items > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const unsigned grid = (unsigned)std::min<int64_t>(items, (int64_t)std::max(1, occ) * std::max(1, sms));

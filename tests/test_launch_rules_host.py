@@ -1,0 +1,38 @@
+"""How the launchers cut a grid into work items (csrc/launch_rules.h, plain host arithmetic compiled here; no GPU)."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SMS = 152
+
+
+@pytest.fixture(scope="module")
+def call(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+
+    def run(expr):
+        src, exe = d / "rule.cpp", d / "rule"
+        src.write_text(f'#include <cstdio>\n#include "launch_rules.h"\n'
+                       f'int main() {{ std::printf("%lld", (long long)({expr})); }}\n')
+        subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_2603_00477_gb300", "csrc"), str(src),
+                        "-o", str(exe)], check=True)
+        return int(subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout)
+    return run
+
+
+# 256^3 in FP64: 64 tiles of 16 x 64 per plane.  Two CTAs per SM: 37 planes are 448 items on 304 CTAs, of which
+# 144 take a second one, so that some SMs work off four (148 planes of work against 120 .. 130 of the others)
+@pytest.mark.parametrize("nz,cols,occ,bad", [(256, 64, 2, 37), (100, 13, 2, 3)])
+def test_streaming_chunks_leave_no_sm_with_one_item_more(call, nz, cols, occ, bad):
+    c = call(f"gbs::stream_planes({nz}, {cols}, {occ}, {SMS})")
+    items = -(-nz // c) * cols
+    rest = items % (occ * SMS)
+    assert c != bad and (items <= occ * SMS or rest == 0 or rest <= 0.8 * SMS or rest > 1.6 * SMS)
+
+
+def test_streaming_chunks_that_stay(call):
+    """Three CTAs per SM (radius 1): 448 items are one wave."""
+    assert call(f"gbs::stream_planes(256, 64, 3, {SMS})") == 37
+    assert 1 <= call(f"gbs::stream_planes(1, 1, 2, {SMS})") <= 1
