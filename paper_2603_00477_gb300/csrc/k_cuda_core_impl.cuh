@@ -147,10 +147,7 @@ stencil_status launch3d_stream(const Plan &p, const void *in, void *out, cudaStr
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu3d_stream launch");
 }
 
-// 3-D, t = 1, FP32: z-marching with rotating partial sums (cu3d_rot).  The
-// run of output planes per work item, cz, is chosen so that the items fill
-// whole rounds of the resident CTAs: the time is ~ rounds x (cz + 2R + a
-// start-up of ~4 planes).
+// 3-D, t = 1, FP32: z-marching with rotating partial sums (cu3d_rot).
 template <int SHAPE, int R, bool VEC>
 stencil_status launch3d_rot(const Plan &p, const void *in, void *out, cudaStream_t st)
 {
@@ -173,15 +170,7 @@ stencil_status launch3d_rot(const Plan &p, const void *in, void *out, cudaStream
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t nz = p.dims[0], cols = (int64_t)tile.tiles_x * tile.tiles_y;
     const int64_t slots = (int64_t)std::max(1, occ) * std::max(1, sms);
-    int64_t cz = nz, best = -1;
-    for (int64_t m = 1; m <= std::min<int64_t>(nz, 512); m++) {
-        const int64_t c = (nz + m - 1) / m, items = ((nz + c - 1) / c) * cols;
-        const int64_t cost = (items + slots - 1) / slots * (c + 2 * R + 4);
-        if (best < 0 || cost < best) {
-            best = cost;
-            cz = c;
-        }
-    }
+    const int64_t cz = rot_planes(nz, cols, R, std::max(1, occ), std::max(1, sms));
     const int64_t items = ((nz + cz - 1) / cz) * cols;
     if (items > 0x7fffffff || cz > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const unsigned grid = (unsigned)std::min<int64_t>(items, slots);

@@ -34,4 +34,25 @@ inline int64_t stream_planes(int64_t nz, int64_t cols, int occ, int sms)
     return best;
 }
 
+// Output planes per work item of the 3-D marching kernel (an item stages 2 r planes more than it
+// writes, and starts up for about four).  Two CTAs on an SM take 1.3 to 1.5 times the time of one per
+// plane (Star-3D3R: 0.97 and 1.48 us), so a sweep of few items is faster with one CTA per SM and longer
+// runs: 128 x 44 x 112, 192 items of two planes 15.3 us, 129 of three 10.8 us (13.2 us with the
+// fixed tiles before); 64^3, 192 items of one 12.9 us, 96 of two 9.8 us.
+inline int64_t rot_planes(int64_t nz, int64_t cols, int r, int occ, int sms)
+{
+    const int64_t slots = (int64_t)occ * sms;
+    int64_t best = nz, best_cost = -1;
+    for (int64_t n = 1; n <= std::min<int64_t>(nz, 512); n++) {
+        const int64_t c = (nz + n - 1) / n, items = (nz + c - 1) / c * cols;
+        const int64_t rounds = items <= sms ? 10 : 14 * ((items + slots - 1) / slots);  // x 1/10
+        const int64_t cost = rounds * (c + 2 * r + 4);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
 }  // namespace gbs

@@ -36,3 +36,16 @@ def test_streaming_chunks_that_stay(call):
     """Three CTAs per SM (radius 1): 448 items are one wave."""
     assert call(f"gbs::stream_planes(256, 64, 3, {SMS})") == 37
     assert 1 <= call(f"gbs::stream_planes(1, 1, 2, {SMS})") <= 1
+
+
+# tiles of a plane as rot_tile cuts it: 128 x 44 x 112 (Star-3D3R) 3, 64^3 (Star-3D3R) 3
+@pytest.mark.parametrize("nz,cols,r,c", [(128, 3, 3, 3), (64, 3, 3, 2)])
+def test_marching_runs_of_a_small_grid_give_an_sm_one_cta(call, nz, cols, r, c):
+    assert call(f"gbs::rot_planes({nz}, {cols}, {r}, 2, {SMS})") == c
+    assert -(-nz // c) * cols <= SMS
+
+
+# 512^3 Star-3D2R, 301 x 417 x 533 Box-3D1R, 256^3 Star-3D3R, a thin grid: two CTAs per SM as before
+@pytest.mark.parametrize("nz,cols,r,c", [(512, 136, 2, 256), (301, 56, 1, 61), (256, 35, 3, 32), (34, 126, 3, 17)])
+def test_marching_runs_that_stay(call, nz, cols, r, c):
+    assert call(f"gbs::rot_planes({nz}, {cols}, {r}, 2, {SMS})") == c
