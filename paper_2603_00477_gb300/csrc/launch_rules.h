@@ -13,7 +13,7 @@ namespace gbs {
 // CTAs that take one item more share an SM as soon as they are more than ~4/5 of the SMs
 // (the block scheduler fills the smaller GPCs twice before the larger ones once): 448
 // items on 304 CTAs are four on some SMs, not three (Box-3D2R FP64 256^3, 37 planes:
-// 18,150 us for four sweeps against 14,580 us with 29 planes and 16,060 us with 64).
+// 18,150 us for four sweeps against 14,030 us with 29 planes and 16,060 us with 64).
 // 64 planes whatever the grid: Box-3D1R FP64 256^3 908 us per sweep, 778 us with 37.
 inline int64_t stream_planes(int64_t nz, int64_t cols, int occ, int sms)
 {
