@@ -5,7 +5,7 @@
 //
 // The band is four thin strips: `band` rows along the top and bottom over the
 // whole width, `band` columns at the left and right of the rows between.  A
-// CTA takes a piece of kBandLen outputs along a strip, stages the piece grown
+// CTA takes a piece of 32 to 128 outputs along a strip, stages the piece grown
 // by t r on every side and runs the t sub-steps in shared memory (ping-pong
 // between two buffers), the last one straight to global memory.  The work is
 // a few thousand points per CTA and bound by latency (t + 1 barriers), so what
@@ -16,39 +16,19 @@
 
 #include "cu_kernels.cuh"
 #include "launch.h"
+#include "launch_rules.h"
 
 namespace gbs {
 namespace {
 
-constexpr int kBandLen = 128;     // outputs of a piece along its strip
 constexpr int kBandThreads = 256;
 constexpr int kBandV = 4;         // outputs of a thread (rows of a column)
 
 struct BandGeom {
-    int64_t ny, nx;        // interior extents
-    int top, bot;          // rows of the top and bottom strips (bot < band only when they would overlap)
-    int left, right;       // columns of the left and right strips
-    int pieces_h;          // pieces of a horizontal strip
-    int pieces_v;          // pieces of a vertical strip
-    int n_h, n_v;          // pieces in all: horizontal first, then vertical
+    int64_t ny, nx;  // interior extents
+    int len;         // outputs of a piece along its strip (band_length)
+    BandPieces p;
 };
-
-BandGeom band_geom(int64_t ny, int64_t nx, int band)
-{
-    BandGeom g{};
-    g.ny = ny;
-    g.nx = nx;
-    g.top = (int)std::min<int64_t>(band, ny);
-    g.bot = (int)std::min<int64_t>(band, ny - g.top);
-    g.left = (int)std::min<int64_t>(band, nx);
-    g.right = (int)std::min<int64_t>(band, nx - g.left);
-    const int64_t mid = ny - g.top - g.bot;
-    g.pieces_h = (int)((nx + kBandLen - 1) / kBandLen);
-    g.pieces_v = (int)((mid + kBandLen - 1) / kBandLen);
-    g.n_h = g.pieces_h * (1 + (g.bot > 0));
-    g.n_v = g.pieces_v * (1 + (g.right > 0));
-    return g;
-}
 
 template <typename T, int SHAPE, int R>
 __global__ void __launch_bounds__(kBandThreads)
@@ -62,19 +42,19 @@ __global__ void __launch_bounds__(kBandThreads)
     int64_t iy0, ix0;
     int BY, BX;
     const int id = blockIdx.x;
-    if (id < g.n_h) {
-        const bool bottom = id >= g.pieces_h;
-        BY = bottom ? g.bot : g.top;
-        iy0 = bottom ? g.ny - g.bot : 0;
-        ix0 = (int64_t)(bottom ? id - g.pieces_h : id) * kBandLen;
-        BX = (int)min((int64_t)kBandLen, g.nx - ix0);
+    if (id < g.p.n_h) {
+        const bool bottom = id >= g.p.h;
+        BY = bottom ? g.p.bot : g.p.top;
+        iy0 = bottom ? g.ny - g.p.bot : 0;
+        ix0 = (int64_t)(bottom ? id - g.p.h : id) * g.len;
+        BX = (int)min((int64_t)g.len, g.nx - ix0);
     } else {
-        const int v = id - g.n_h;
-        const bool right = v >= g.pieces_v;
-        BX = right ? g.right : g.left;
-        ix0 = right ? g.nx - g.right : 0;
-        iy0 = g.top + (int64_t)(right ? v - g.pieces_v : v) * kBandLen;
-        BY = (int)min((int64_t)kBandLen, g.ny - g.bot - iy0);
+        const int v = id - g.p.n_h;
+        const bool right = v >= g.p.v;
+        BX = right ? g.p.right : g.p.left;
+        ix0 = right ? g.nx - g.p.right : 0;
+        iy0 = g.p.top + (int64_t)(right ? v - g.p.v : v) * g.len;
+        BY = (int)min((int64_t)g.len, g.ny - g.p.bot - iy0);
     }
     const int64_t Ey = g.ny + 2 * R;
     const int H = BY + 2 * t * R, W = BX + 2 * t * R;
@@ -151,13 +131,17 @@ stencil_status launch_band_n(const Plan &p, const void *in, void *out, int t, in
     using Wt = cu::Weights<T, cu::Taps<SHAPE, 2, R>::K>;
     Wt wt;
     for (int k = 0; k < cu::Taps<SHAPE, 2, R>::K; k++) wt.w[k] = (T)p.w[k];
-    const BandGeom g = band_geom(p.dims[1], p.dims[2], band);
-    const size_t smem = (size_t)(band + 2 * t * R) * (kBandLen + 2 * t * R) * sizeof(T) * 2;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    BandGeom g{p.dims[1], p.dims[2], band_length(p.dims[1], p.dims[2], band, std::max(1, sms)), {}};
+    g.p = band_pieces(g.ny, g.nx, band, g.len);
+    const size_t smem = (size_t)(band + 2 * t * R) * (g.len + 2 * t * R) * sizeof(T) * 2;
     if (smem > 227 * 1024) return fail(STENCIL_ERR_UNSUPPORTED, "CUDA-core band does not fit in shared memory");
     auto kern = cu2d_band<T, SHAPE, R>;
     stencil_status s = ensure_smem((const void *)kern, smem);
     if (s != STENCIL_OK) return s;
-    const cudaError_t e = launch_chained(kern, (unsigned)(g.n_h + g.n_v), kBandThreads, smem, st, (const T *)in,
+    const cudaError_t e = launch_chained(kern, (unsigned)(g.p.n_h + g.p.n_v), kBandThreads, smem, st, (const T *)in,
                                          (T *)out, wt, p.ext[2], t, g);
     if (e == cudaSuccess) note_launch();
     return e == cudaSuccess ? STENCIL_OK : cuda_fail(e, "cu2d_band launch");

@@ -49,3 +49,50 @@ def test_marching_runs_of_a_small_grid_give_an_sm_one_cta(call, nz, cols, r, c):
 @pytest.mark.parametrize("nz,cols,r,c", [(512, 136, 2, 256), (301, 56, 1, 61), (256, 35, 3, 32), (34, 126, 3, 17)])
 def test_marching_runs_that_stay(call, nz, cols, r, c):
     assert call(f"gbs::rot_planes({nz}, {cols}, {r}, 2, {SMS})") == c
+
+
+# a small grid's band is cut into more pieces; pieces never number more than the SMs for being short
+@pytest.mark.parametrize("ny,nx,band,length", [(300, 200, 3, 32), (100, 100, 9, 32), (1500, 1400, 6, 64), (16384, 16384, 6, 128),
+                                               (1, 300, 4, 32), (2000, 2600, 4, 64)])
+def test_band_pieces_of_a_small_grid(call, ny, nx, band, length):
+    got = call(f"gbs::band_length({ny}, {nx}, {band}, {SMS})")
+    assert got == length
+
+
+@pytest.mark.parametrize("ny,nx,band", [(1, 1, 3), (2, 300, 3), (300, 2, 5), (7, 9, 4), (130, 259, 6), (33, 32, 8)])
+@pytest.mark.parametrize("length", [32, 64, 128])
+def test_band_pieces_cover_the_band_once(tmp_path, ny, nx, band, length):
+    """Every interior point nearer than `band` to the boundary is in exactly one piece, as the kernel reads them."""
+    prog = f"""
+#include <cstdio>
+#include <vector>
+#include "launch_rules.h"
+int main() {{
+    const gbs::BandPieces g = gbs::band_pieces({ny}, {nx}, {band}, {length});
+    std::vector<int> seen({ny} * {nx}, 0);
+    for (int id = 0; id < g.n_h + g.n_v; id++) {{
+        long y0, x0, by, bx;
+        if (id < g.n_h) {{
+            const bool b = id >= g.h;
+            by = b ? g.bot : g.top; y0 = b ? {ny} - g.bot : 0;
+            x0 = (long)(b ? id - g.h : id) * {length}; bx = std::min<long>({length}, {nx} - x0);
+        }} else {{
+            const int v = id - g.n_h; const bool r = v >= g.v;
+            bx = r ? g.right : g.left; x0 = r ? {nx} - g.right : 0;
+            y0 = g.top + (long)(r ? v - g.v : v) * {length}; by = std::min<long>({length}, {ny} - g.bot - y0);
+        }}
+        for (long y = y0; y < y0 + by; y++) for (long x = x0; x < x0 + bx; x++) seen[y * {nx} + x]++;
+    }}
+    int bad = 0;
+    for (int y = 0; y < {ny}; y++) for (int x = 0; x < {nx}; x++) {{
+        const bool in = y < {band} || x < {band} || {ny} - 1 - y < {band} || {nx} - 1 - x < {band};
+        bad += seen[y * {nx} + x] != (in ? 1 : 0);
+    }}
+    std::printf("%d", bad);
+}}
+"""
+    src, exe = tmp_path / "b.cpp", tmp_path / "b"
+    src.write_text(prog)
+    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_2603_00477_gb300", "csrc"), str(src), "-o",
+                    str(exe)], check=True)
+    assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout == "0"
