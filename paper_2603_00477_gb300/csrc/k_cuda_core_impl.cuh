@@ -72,7 +72,8 @@ stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStr
         // a tile asked for by option or picked by the autotuner runs the tiled kernel
         int def[3];
         cu_default_tile(p, p.t, def);
-        if (t <= 2 && tile[1] == def[1] && tile[2] == def[2]) {
+        if (t <= 2 && tile[1] == def[1] && tile[2] == def[2] &&
+            !tiles_beat_march(SHAPE, R, t, p.dims[1], p.dims[2], tile[1], tile[2])) {
             const bool vec = p.ext[2] % 4 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0 &&
                              reinterpret_cast<uintptr_t>(out) % 16 == 0;
             if (t == 1)

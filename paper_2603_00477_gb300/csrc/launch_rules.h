@@ -6,6 +6,16 @@
 
 namespace gbs {
 
+// Where the tiled 2-D FP32 kernel is faster than the marching one although that has the depth: box r = 3 at t = 1
+// (shape 0) on grids that the tile divides, where every tile takes the tiled kernel's fixed-strip sub-step.  A
+// warp of the marching kernel walks six rows of halo at 196 FMAs a row for its few rows.  Marching and
+// tiled, one sweep: 256^2 6.6 and 4.3 us, 512^2 8.8 and 5.1, 1024^2 10.2 and 9.3, 2048^2 19.2 and 16.6,
+// 4096^2 51.7 and 55.7; 512 x 90, not divided, 5.1 and 7.1.
+inline bool tiles_beat_march(int shape, int r, int t, int64_t ny, int64_t nx, int tile_y, int tile_x)
+{
+    return shape == 0 && r == 3 && t == 1 && ny % tile_y == 0 && nx % tile_x == 0 && ny * nx <= 6000000;
+}
+
 // Output planes per work item of the 3-D streaming kernel (`cols` tiles of a plane
 // side by side, `occ` resident CTAs per SM).  The FMA pipe is the bound and an SM's
 // CTAs share it, so a sweep takes about (items of the busiest SM) x (planes + a start-up

@@ -96,3 +96,10 @@ int main() {{
     subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_2603_00477_gb300", "csrc"), str(src), "-o",
                     str(exe)], check=True)
     assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout == "0"
+
+
+@pytest.mark.parametrize("args,tiles", [("0, 3, 1, 512, 512, 16, 32", 1), ("0, 3, 1, 2048, 2048, 64, 128", 1),
+                                        ("0, 3, 1, 4096, 4096, 64, 128", 0), ("0, 3, 1, 512, 90, 16, 32", 0),
+                                        ("1, 3, 1, 512, 512, 16, 32", 0), ("0, 2, 1, 512, 512, 16, 32", 0)])
+def test_tiled_or_marching(call, args, tiles):
+    assert call(f"gbs::tiles_beat_march({args})") == tiles
