@@ -77,6 +77,7 @@ struct Tiles {
     int xshift;      // FP32: the tile grid starts xshift columns further left so that every
                      // staged window begins on a 16-byte boundary (then vec16 = 1)
     int vec16;       // stage interior tiles with 16-byte copies
+    int next_early;  // chain_next at the start (next_sweep_early)
 };
 
 // Asynchronous global -> shared copy of one element (cp.async, L1-allocating);
@@ -96,10 +97,8 @@ __device__ __forceinline__ void cp_async_elem(void *smem_dst, const void *gmem_s
 // blocks take their places (chain_next) as soon as its own have all started, or,
 // where a sweep is bound by the FMA pipes, when their work is done: blocks placed
 // earlier pile up on the SMs that finish first.  (FP64 Box-2D3R on 600 x 500, ten
-// sweeps: 296 us unchained, 403 us with chain_next at the start.  FP32 tiles, eight
-// sweeps: Star-2D6R 2048 x 2044 508 us unchained, 551 early, 488 late; Star-2D7R t = 3
-// 1068, 1151, 1061; up to radius 5 early is never slower than unchained: Star-2D5R
-// 1000 x 1003 122, 100, 105.)
+// sweeps: 296 us unchained, 403 us with chain_next at the start.)  The tiled 2-D kernel
+// has either (next_sweep_early).
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -526,8 +525,7 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
                const __grid_constant__ Weights<T, Taps<SHAPE, 2, R>::K> wt, int64_t Ey, int64_t Ex, int BY, int BX,
                int t, const Tiles tiles, int ntiles)
 {
-    constexpr bool kNextEarly = sizeof(T) == 4 && R <= 5;
-    if constexpr (kNextEarly) chain_next();
+    if (tiles.next_early) chain_next();
     chain_wait();
     constexpr int KT = Taps<SHAPE, 2, R>::K;
     constexpr bool kSmemW = sizeof(T) == 8;
@@ -706,7 +704,7 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && R <= 3) ? 3 : 2)
         cur ^= 1;
     }
     cp_async_wait_group<0>();
-    if constexpr (!kNextEarly) chain_next();
+    if (!tiles.next_early) chain_next();
 }
 
 // ---------------------------------------------------------------------------

@@ -111,6 +111,7 @@ stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStr
     if (ntiles > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
     const int64_t resident = (int64_t)std::max(1, occ_blocks) * std::max(1, sms);
     const unsigned grid = (unsigned)std::min<int64_t>(ntiles, resident);
+    tiles.next_early = next_sweep_early(sizeof(T) == 8, R, t, ntiles, resident);
     const cudaError_t e = launch_chained(kern, grid, cu::kThreads, smem, st, (const T *)in, (T *)out, wt,
                                          p.ext[1], p.ext[2], BY, BX, t, tiles, (int)ntiles);
     if (e == cudaSuccess) note_launch();

@@ -16,6 +16,18 @@ inline bool tiles_beat_march(int shape, int r, int t, int64_t ny, int64_t nx, in
     return shape == 0 && r == 3 && t == 1 && ny % tile_y == 0 && nx % tile_x == 0 && ny * nx <= 6000000;
 }
 
+// When a sweep of the tiled 2-D kernel lets the blocks of the next sweep in (chained launches): at its start, or when
+// a block's work is done.  Blocks let in early take the slots of the blocks that finish first, the next
+// sweep's blocks with one tile more among them, and share those SMs; where the FMA pipe is the bound (FP64, and
+// FP32 from radius 4 on) that costs more than the head start gives, unless one-step sweeps have three tiles
+// per block or more.  Eight sweeps, unchained / early / late: Box-2D4R FP32 1440 x 2560 189 / 218 / 169 us, Star-2D6R
+// 1440 x 2560 300 / 326 / 282, Star-2D7R t = 3 2048 x 2048 1043 / 1118 / 1033, Star-2D6R 3000 x 3000 826 / 705 / 806,
+// Box-2D4R 3000 x 3000 439 / 392 / 419.
+inline bool next_sweep_early(bool f64, int r, int t, int64_t tiles, int64_t resident)
+{
+    return !f64 && (r <= 3 || (t == 1 && tiles >= 3 * resident));
+}
+
 // Output planes per work item of the 3-D streaming kernel (`cols` tiles of a plane
 // side by side, `occ` resident CTAs per SM).  The FMA pipe is the bound and an SM's
 // CTAs share it, so a sweep takes about (items of the busiest SM) x (planes + a start-up

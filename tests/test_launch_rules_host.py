@@ -103,3 +103,10 @@ int main() {{
                                         ("1, 3, 1, 512, 512, 16, 32", 0), ("0, 2, 1, 512, 512, 16, 32", 0)])
 def test_tiled_or_marching(call, args, tiles):
     assert call(f"gbs::tiles_beat_march({args})") == tiles
+
+
+@pytest.mark.parametrize("args,early", [("true, 3, 1, 100000, 456", 0), ("false, 3, 3, 500, 456", 1),
+                                        ("false, 4, 1, 460, 304", 0), ("false, 6, 1, 1128, 304", 1),
+                                        ("false, 6, 2, 1128, 304", 0), ("false, 7, 3, 552, 304", 0)])
+def test_when_the_next_sweep_is_let_in(call, args, early):
+    assert call(f"gbs::next_sweep_early({args})") == early
