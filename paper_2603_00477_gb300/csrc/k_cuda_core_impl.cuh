@@ -109,6 +109,7 @@ stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStr
     tiles.ntx = (int)((p.dims[2] + tiles.xshift + BX - 1) / BX);
     const int64_t ntiles = (p.dims[1] + BY - 1) / BY * tiles.ntx;
     if (ntiles > 0x7fffffff) return fail(STENCIL_ERR_UNSUPPORTED, "too many tiles");
+    if (sizeof(T) == 8) occ_blocks = f64_tile_ctas(ntiles, std::max(1, occ_blocks), std::max(1, sms));
     const int64_t resident = (int64_t)std::max(1, occ_blocks) * std::max(1, sms);
     const unsigned grid = (unsigned)std::min<int64_t>(ntiles, resident);
     tiles.next_early = next_sweep_early(sizeof(T) == 8, R, t, ntiles, resident);

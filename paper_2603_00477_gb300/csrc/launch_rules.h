@@ -28,26 +28,39 @@ inline bool next_sweep_early(bool f64, int r, int t, int64_t tiles, int64_t resi
     return !f64 && (r <= 3 || (t == 1 && tiles >= 3 * resident));
 }
 
-// Output planes per work item of the 3-D streaming kernel (`cols` tiles of a plane
-// side by side, `occ` resident CTAs per SM).  The FMA pipe is the bound and an SM's
-// CTAs share it, so a sweep takes about (items of the busiest SM) x (planes + a start-up
-// worth one plane).  Up to one wave the CTAs are spread evenly; beyond it the persistent
-// CTAs that take one item more share an SM as soon as they are more than ~4/5 of the SMs
-// (the block scheduler fills the smaller GPCs twice before the larger ones once): 448
-// items on 304 CTAs are four on some SMs, not three (Box-3D2R FP64 256^3, 37 planes:
-// 18,150 us for four sweeps against 14,030 us with 29 planes and 16,060 us with 64).
-// 64 planes whatever the grid: Box-3D1R FP64 256^3 908 us per sweep, 778 us with 37.
+// Items of the busiest SM when persistent CTAs, `occ` resident per SM, work off `items`.  Up to one wave the CTAs
+// are spread evenly; beyond it those that take one item more share an SM as soon as they are more than ~4/5 of
+// the SMs (the block scheduler fills the smaller GPCs twice before the larger ones once): 448 items on 304 CTAs
+// are four on some SMs, not three.
+inline int64_t busiest_items(int64_t items, int occ, int sms)
+{
+    const int64_t wave = (int64_t)occ * sms, full = items / wave, rest = items % wave;
+    if (full == 0) return (rest + sms - 1) / sms;
+    return occ * full + (rest > 0 ? std::min<int64_t>(occ, (5 * rest + 4 * sms - 1) / (4 * sms)) : 0);
+}
+
+// Persistent CTAs per SM of the tiled 2-D kernel in FP64, at most `occ`: the FP64 pipe is the bound and two CTAs fill
+// it, so the fewest items on the busiest SM count.  Box-2D5R 480 x 640: 600 tiles on 456 CTAs are five on some
+// SMs (640 us for eight sweeps), on 304 CTAs four (547 us).
+inline int f64_tile_ctas(int64_t tiles, int occ, int sms)
+{
+    int best = occ;
+    for (int o = occ - 1; o >= 2; o--)
+        if (busiest_items(tiles, o, sms) < busiest_items(tiles, best, sms)) best = o;
+    return best;
+}
+
+// Output planes per work item of the 3-D streaming kernel (`cols` tiles of a plane side by side, `occ` resident
+// CTAs per SM).  The FMA pipe is the bound and an SM's CTAs share it, so a sweep takes about (items of the busiest
+// SM) x (planes + a start-up worth one plane).  Box-3D2R FP64 256^3, four sweeps: 18,150 us with 37 planes (448
+// items counted as three on the busiest of 152 SMs), 14,030 us with 29, 16,060 us with 64.  64 planes whatever the grid:
+// Box-3D1R FP64 256^3 908 us per sweep, 778 us with 37.
 inline int64_t stream_planes(int64_t nz, int64_t cols, int occ, int sms)
 {
-    const int64_t wave = (int64_t)occ * sms;
     int64_t best = nz, best_cost = -1;
     for (int64_t n = 1; n <= std::min<int64_t>(nz, 64); n++) {
-        const int64_t c = (nz + n - 1) / n, items = (nz + c - 1) / c * cols;
-        const int64_t full = items / wave, rest = items % wave;
-        int64_t busiest = occ * full;
-        if (full == 0) busiest = (rest + sms - 1) / sms;
-        else if (rest > 0) busiest += std::min<int64_t>(occ, (5 * rest + 4 * sms - 1) / (4 * sms));
-        const int64_t cost = busiest * (c + 1);
+        const int64_t c = (nz + n - 1) / n;
+        const int64_t cost = busiest_items((nz + c - 1) / c * cols, occ, sms) * (c + 1);
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best = c;

@@ -110,3 +110,10 @@ def test_tiled_or_marching(call, args, tiles):
                                         ("false, 6, 2, 1128, 304", 0), ("false, 7, 3, 552, 304", 0)])
 def test_when_the_next_sweep_is_let_in(call, args, early):
     assert call(f"gbs::next_sweep_early({args})") == early
+
+
+# 600 tiles: three CTAs per SM leave some SMs with five, two with four; the others keep what the occupancy allows
+@pytest.mark.parametrize("tiles,occ,ctas", [(600, 3, 2), (512, 3, 3), (65536, 3, 3), (100, 3, 3), (456, 3, 3), (600, 2, 2),
+                                            (600, 1, 1)])
+def test_fp64_tiles_per_sm(call, tiles, occ, ctas):
+    assert call(f"gbs::f64_tile_ctas({tiles}, {occ}, {SMS})") == ctas
