@@ -32,7 +32,7 @@ struct BandGeom {
 
 template <typename T, int SHAPE, int R>
 __global__ void __launch_bounds__(kBandThreads)
-    cu2d_band(const T *__restrict__ in, T *__restrict__ out,
+    cu2d_band(const T *in, T *__restrict__ out,
               const __grid_constant__ cu::Weights<T, cu::Taps<SHAPE, 2, R>::K> wt, int64_t Ex, int t,
               const BandGeom g)
 {
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kBandThreads)
     for (int e = tid; e < H * W; e += kBandThreads) {
         const int y = e / W, x = e - (e / W) * W;
         const int64_t gy = Y0 + y, gx = X0 + x;
-        src[e] = (gy >= 0 && gy < Ey && gx >= 0 && gx < Ex) ? in[gy * Ex + gx] : T(0);
+        src[e] = (gy >= 0 && gy < Ey && gx >= 0 && gx < Ex) ? __ldcg(in + gy * Ex + gx) : T(0);
     }
     __syncthreads();
     for (int s = 1; s <= t; ++s) {

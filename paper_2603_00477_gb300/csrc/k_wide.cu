@@ -527,8 +527,8 @@ __device__ __forceinline__ void block_sweep(const float *__restrict__ in, float 
                             sh |= s << (2 * u);
                             if (i0 + u * kLoaders < items) {
                                 const float4 *a4 = reinterpret_cast<const float4 *>(q - s);
-                                v[u] = __ldg(a4);
-                                if (s) v[U + u] = __ldg(a4 + 1);
+                                v[u] = ld_chained(a4);
+                                if (s) v[U + u] = ld_chained(a4 + 1);  // in L1: the next lane's first word
                             }
                             next();
                         }

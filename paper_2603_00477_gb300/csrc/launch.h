@@ -74,7 +74,10 @@ stencil_status occupancy(const void *func, int threads, size_t smem, int *blocks
 // run (programmatic stream serialisation), which takes the gap between dependent
 // launches out of a run of short sweeps.  The attribute also holds under stream
 // capture.  The kernel in front must be a kernel of the same run (the halo copy or
-// a sweep).
+// a sweep).  Its input is not constant for the lifetime of the chained kernel, whose
+// blocks are resident while it is still written: after chain_wait() it is read with
+// cp.async, __ldcg or ld_chained, never with __ldg or through a `const __restrict__`
+// pointer that the compiler may read the same way.
 // Measured, unchained before: Star-2D1R FP64 512^2, 10 steps 86 -> 56 us;
 // Star-2D2R FP32 1021 x 1531, 20 steps 107 -> 87 us; Box-2D3R FP64 230 x 310,
 // 10 steps 127 -> 103 us; Star-3D1R FP32 64 x 65 x 66, 6 steps 41 -> 31 us;

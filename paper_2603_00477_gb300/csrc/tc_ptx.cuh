@@ -111,6 +111,14 @@ __device__ __forceinline__ void mma_commit(uint64_t *mbar)
                  : "memory");
 }
 
+// 16 bytes of a chained kernel's input (launch_chained), through L1 but not the read-only path.
+__device__ __forceinline__ float4 ld_chained(const float4 *p)
+{
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
 // True in exactly one lane of a converged warp (always the same one).
 __device__ __forceinline__ uint32_t elect_lane()
 {
