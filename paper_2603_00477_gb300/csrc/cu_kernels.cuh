@@ -130,13 +130,13 @@ __device__ __forceinline__ void static_for(F &&f)
 // touches, whose partial sums rotate through 2R+1 register slots.  The row
 // loop is unrolled by 2R+1, so every slot index and weight index is a
 // compile-time constant and no FMA carries a condition; output row jj is
-// complete after input row jj + 2R and is stored from its slot.  When the
-// whole region is interior the stores skip the boundary tests.
+// complete after input row jj + 2R and is stored from its slot.  `fast`: the
+// whole region is interior and the stores skip the boundary tests.
 template <int SHAPE, int R, int D, typename WT>
 __device__ __forceinline__ void f32_substep(const float *__restrict__ src, float *__restrict__ dst,
                                             float *__restrict__ out, const WT &wt, int W, int H, int lo, int hiY,
                                             int hiX, int64_t Y0, int64_t X0, int64_t Ey, int64_t Ex, bool last,
-                                            bool all_interior, int band)
+                                            bool fast)
 {
     constexpr int NS = 2 * R + 1;      // rotating slots
     constexpr int NV = 2 * R + 2 + D;  // window values per row
@@ -147,9 +147,6 @@ __device__ __forceinline__ void f32_substep(const float *__restrict__ src, float
     // redundant work), enough of them to give every thread work
     const int nstrips = max(1, min((ch + 15) / 16, (int)((blockDim.x + npairs - 1) / npairs)));
     const int S = (ch + nstrips - 1) / nstrips;
-    const int64_t ny = Ey - 2 * R, nx = Ex - 2 * R;
-
-    const bool fast = all_interior && band == 0;
     auto store = [&](int y, int x, float v0, float v1, bool second) {
         if (fast) {
             if (last) {
@@ -182,12 +179,7 @@ __device__ __forceinline__ void f32_substep(const float *__restrict__ src, float
             const bool interior = rowint && gxh >= R && gxh < Ex - R;
             const float val = h ? v1 : v0;
             if (last) {
-                bool keep = interior;
-                if (band > 0) {
-                    const int64_t iy = gy - R, ix = gxh - R;
-                    keep = keep && (iy < band || ix < band || ny - 1 - iy < band || nx - 1 - ix < band);
-                }
-                if (keep) out[gy * Ex + gxh] = val;
+                if (interior) out[gy * Ex + gxh] = val;
             } else {
                 dst[y * W + x + h] = interior ? val : src[y * W + x + h];
             }

@@ -207,10 +207,10 @@ __device__ void run_item(const GridDev &G, const T *__restrict__ wg, const T *sr
             const bool all_int = Y0 + lo >= R && Y0 + hiY <= Ey - R && X0 + lo >= R && X0 + hiX <= Ex - R;
             if (((lo - R) & 1) == 0)
                 cu::f32_substep<SHAPE, R, 0>(src, dst, dst_g, wrs, P, H, lo, hiY, hiX, Y0, X0, Ey, Ex, last,
-                                                all_int, 0);
+                                             all_int);
             else
                 cu::f32_substep<SHAPE, R, 1>(src, dst, dst_g, wrs, P, H, lo, hiY, hiX, Y0, X0, Ey, Ex, last,
-                                                all_int, 0);
+                                             all_int);
             __syncthreads();
             T *tmp = src;
             src = dst;

@@ -66,8 +66,7 @@ stencil_status launch2d(const Plan &p, const void *in, void *out, int t, cudaStr
     using Wt = cu::Weights<T, cu::Taps<SHAPE, 2, R>::K>;
     Wt wt;
     for (int k = 0; k < cu::Taps<SHAPE, 2, R>::K; k++) wt.w[k] = (T)p.w[k];
-    int tile[3] = {p.tile[0], p.tile[1], p.tile[2]};
-    if (p.path != STENCIL_PATH_CUDA_CORE) cu_default_tile(p, t, tile);
+    const int *tile = p.tile;
     if constexpr (sizeof(T) == 4 && R <= 3) {
         // a tile asked for by option or picked by the autotuner runs the tiled kernel
         int def[3];
@@ -200,8 +199,7 @@ stencil_status launch3d(const Plan &p, const void *in, void *out, int t, cudaStr
     using Wt = cu::Weights<T, cu::Taps<SHAPE, 3, R>::K>;
     Wt wt;
     for (int k = 0; k < cu::Taps<SHAPE, 3, R>::K; k++) wt.w[k] = (T)p.w[k];
-    int tile[3] = {p.tile[0], p.tile[1], p.tile[2]};
-    if (p.path != STENCIL_PATH_CUDA_CORE) cu_default_tile(p, t, tile);
+    const int *tile = p.tile;
     const int BZ = tile[0], BY = tile[1], BX = tile[2];
     const size_t Z = BZ + 2 * t * R, H = BY + 2 * t * R, W = BX + 2 * t * R;
     const size_t smem =

@@ -80,17 +80,6 @@ __device__ __forceinline__ void fence_proxy_async_smem()
 
 // ---- MMA -------------------------------------------------------------------
 // D[tmem] (+)= A[smem] * B[smem]; accumulate != 0 keeps the old D.
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                         uint32_t accumulate)
 {
@@ -196,49 +185,10 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *mbar, uint32_t phase)
     return ok != 0;
 }
 
-// Bounded wait: gives up after max_tries polls (each poll may itself block
-// for a hardware-defined time slice) and returns false.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *mbar, uint32_t phase, uint32_t max_tries)
-{
-    for (uint32_t i = 0; i < max_tries; ++i)
-        if (mbar_try_wait(mbar, phase)) return true;
-    return false;
-}
-
 // Arrive (once per calling thread) on an mbarrier.
 __device__ __forceinline__ void mbar_arrive(uint64_t *mbar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
-}
-
-// Arrive once on an mbarrier and add `bytes` to the transaction count its
-// current phase waits for (the bytes of the TMA copies that complete on it).
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *mbar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)), "r"(bytes)
-                 : "memory");
-}
-
-// ---- TMA -------------------------------------------------------------------
-// Tiled 2-D copy of the box at element coordinates (x, y) of the tensor map
-// `tmap` (a __grid_constant__ kernel parameter) into shared memory at dst
-// (128-byte aligned); completes `bytes` of the transaction count of mbar.
-// Out-of-range elements are written as zeros.  x times the element size must
-// be a multiple of 16 bytes.
-__device__ __forceinline__ void tma_load_2d(void *dst, const void *tmap, int x, int y, uint64_t *mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-            "r"(smem_u32(dst)),
-        "l"(tmap), "r"(x), "r"(y), "r"(smem_u32(mbar))
-        : "memory");
-}
-
-// Barrier among a subset of the CTA's warps (named barrier `id`, `count`
-// threads, a multiple of 32).
-__device__ __forceinline__ void named_bar_sync(int id, int count)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
 // ---- TMEM -> registers -----------------------------------------------------
