@@ -89,7 +89,9 @@ typedef enum {
  * FP16 tensor cores with exact FP32 sums, and the levels are recombined in
  * 64-bit integers: FP64 accuracy (a few units of 2^-53 per sweep,
  * normwise).  F16 / F16X3 (FP32 grids, tensor-core path): FP16 operands with
- * a power-of-two scale per staged tile (and one for the composite weights),
+ * a power-of-two scale per staged tile (and one for the composite weights)
+ * that puts the tile's largest |x| in [2^14, 65504], so that values down to
+ * 2^-28 of it keep 11 bits and down to 2^-17 of it 22 bits as hi + lo,
  * one product (F16: 11 significant bits, TF32's) or hi + lo parts with three
  * products (F16X3: 22 bits, TF32x3's), FP32 accumulation; a kind::f16 MMA
  * takes K = 16 per instruction against TF32's 8.  3-D grids take the
@@ -125,16 +127,23 @@ typedef struct {
     int path;             /* stencil_path actually used                      */
     int precision;        /* stencil_precision actually used                 */
     int t;                /* fusion depth                                    */
-    int tile[3];          /* output tile per CTA, slowest axis first         */
+    int tile[3];          /* output tile per CTA, slowest axis first; native
+                             FP32 at t <= 2 with r <= 3 (2-D) and t = 1 (3-D)
+                             cuts the grid at launch instead, unless a 2-D
+                             tile was set by option or by the autotuner      */
     int K;                /* points of the pattern                           */
     int K_fused;          /* K^(t), points of the composite kernel           */
     double alpha;         /* K^(t)/(tK)  (Eq. 9); 1 on the CUDA-core path    */
-    double sparsity;      /* S of the MMA tiles (useful/issued); 1 on CU     */
+    double sparsity;      /* S of the MMA tiles (useful/issued) of the line
+                             form (stencil_tc_layout); 1 on CU               */
     double beta;          /* products issued per useful product (1 or 3)     */
     double intensity;     /* FLOP/byte of the chosen path (Eq. 8 / Eq. 12)   */
     double ridge;         /* P/B of the unit that runs the path              */
     int scenario;         /* 1..4 (Sec. 4.1) of CU vs TC at this t           */
     int memory_bound;     /* 1 if the chosen path is below its ridge         */
+    /* The dispatcher's model.  Its instruction roofs for 2-D FP32 grids
+     * were measured on earlier kernels; the present ones run up to about twice
+     * as fast (stencil_plan_autotune measures). */
     double predicted_gstencils;    /* point-updates/s / 1e9 at the roof      */
     double predicted_cu_gstencils; /* CU path at this t                      */
     double predicted_tc_gstencils; /* TC path at this t (0 if not available) */
@@ -164,13 +173,16 @@ typedef struct {
 
 /* Geometry of the tensor-core Toeplitz operands for one fusion depth
  * (paper Sec. 2.2: the stencil recast as an MMA over zero-padded banded
- * matrices).  For line a (row a of the composite kernel w^(t), a = -R..R)
- * the B operand is B_a[k][n] = w^(t)[a][k - n - R] for |k - n - R| <= R,
- * else 0, k in [0, kext), n in [0, n_tile); the MMAs issue the K blocks
- * kb_lo[a]..kb_hi[a] of k_inst columns each. */
+ * matrices), in line form.  For line a (row a of the composite kernel w^(t),
+ * a = -R..R) the B operand is B_a[k][n] = w^(t)[a][k - n - R] for
+ * |k - n - R| <= R, else 0, k in [0, kext), n in [0, n_tile); the form takes
+ * the K blocks kb_lo[a]..kb_hi[a] of k_inst columns each.  The FP64 kernels
+ * issue these MMAs.  The 2-D FP32 kernels issue the same products as blocks of
+ * 16 x 8 outputs, (16 + 2R)/2 * ceil((8 + 2R)/c) MMAs per block and product
+ * (c = 8 values per 16 bytes, TF32: 4), fewer than the line form's. */
 typedef struct {
     int R;          /* fused radius t*r                          */
-    int n_tile;     /* MMA N: output columns per accumulator     */
+    int n_tile;     /* output columns per Toeplitz block         */
     int k_inst;     /* MMA K per instruction                     */
     int kext;       /* padded K extent of one line               */
     int nkb;        /* kext / k_inst                             */
@@ -378,7 +390,8 @@ typedef struct stencil_batch stencil_batch;
  * dtype, run together: one persistent launch whose CTAs pull (grid, tile,
  * sweep) work items from a device queue; an item of sweep s waits (bounded)
  * for every tile of sweep s-1 of its grid.  Each grid gets the CUDA-core
- * fusion depth and tile the model picks for it (t = 0) or the given t.
+ * fusion depth the model picks for it (t = 0) or the given t, and a tile that
+ * also depends on the other grids of the batch (stencil_batch_info).
  * Host only.  INVALID_ARG for bad arguments, UNSUPPORTED for r > 3. */
 stencil_status stencil_batch_create(stencil_batch **batch, int n, const stencil_grid_desc *grids,
                                     stencil_dtype dtype, int t);
@@ -447,7 +460,8 @@ typedef struct {
  * for size classes >= 3 when the batch precision allows (FP64 batches, or
  * FP32 with precision other than "native"), the dense and sparse
  * tensor-core paths (t = 1..4) -- by the model, measures the model's best
- * four of each path and the current choice on the class's grids alone (`reps` timed runs of
+ * four of each path and the current choice on the class's grids alone, in the
+ * kernel that the whole batch runs (`reps` timed runs of
  * `steps` steps after one untimed run, CUDA events on `stream`, inputs
  * ins/outs as for stencil_batch_run; outputs are overwritten), and gives every
  * grid of the class the fastest.  Writes up to max_results rows (results may

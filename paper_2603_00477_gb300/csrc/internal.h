@@ -44,7 +44,7 @@ ModelOut model_eval(int shape, int d, int r, int t, int D, double S, double beta
 
 stencil_peaks peaks();  // a copy of the process-wide table (thread safe)
 
-// ---- tensor-core tile geometry (host view of what the TC kernels issue) ----
+// ---- tensor-core tile geometry (the line form, tc_layout.h) ----
 struct TcGeometry {
     bool available = false;
     int n_tile = 0;      // MMA N (output columns per accumulator)

@@ -7,10 +7,17 @@
 // every tile of sweep s-1 of g has been counted done (bounded spin); because
 // every item it waits for has a smaller index and was therefore already
 // taken by a running CTA, the wait always ends without any co-residency
-// assumption.  Each item stages its tile grown by t*r (L2-coherent loads:
-// other CTAs of the same launch produced the data), runs the grid's t
-// sub-steps on CUDA cores in shared memory (the same temporal blocking as
-// cu2d_sweep) and writes the tile.  Sweep-0 items also copy the halo cells
+// assumption.  An item is a shared-memory tile (staged grown by t*r with loads
+// from L2, the grid's t sub-steps in shared memory as in cu2d_sweep) or, in FP32
+// where the marching kernel has the depth and march_pays says so, a group of
+// warp strips (cu::march_strip).  Memory order: other CTAs of the same launch
+// wrote the data of an item of sweep s > 0.  A CTA's writes are followed by
+// __threadfence and the count of its item (by thread 0, behind a barrier); thread 0
+// of the reading CTA loads that counter with ld.acquire.gpu, and the barrier after
+// it orders the other threads' loads behind.  The tiles' loads go to L2 anyway; the
+// strips' cp.async go through L1 and depend on the acquire: a line that the SM read
+// earlier is dropped by it, so it must not become a relaxed or volatile load, and every
+// item of sweep s > 0 has to pass it.  Sweep-0 items also copy the halo cells
 // nearest to their tile from `in` to the grid's output and ping-pong buffers.
 // On a wait that runs out, the CTA sets the abort word and every CTA leaves.
 #include <algorithm>
@@ -77,8 +84,8 @@ __device__ __forceinline__ T ld_l2(const T *p)
 // down them on its own (cu::march_strip), so an item has no barrier inside.  The
 // shared-memory tiles below (the other depths and types) stage, wait and compute
 // in phases: a batch of 64 grids of 64 .. 4096 points a side, 20 steps, took 8.2 ms
-// with them and 3.2 ms here (3.35 with scalar FMAs: the weights are in registers,
-// so the packed ones only save issue slots).
+// with them and 2.9 ms here (scalar FMAs instead of packed ones 5 % more: the weights
+// are in registers, so the packed ones only save issue slots).
 template <int SHAPE, int R, int T, bool VEC>
 __device__ __noinline__ void march_tile(const GridDev &G, const float *__restrict__ wg, const float *src_g,
                                         float *dst_g, int tile, float *smem)

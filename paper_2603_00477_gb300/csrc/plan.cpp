@@ -299,12 +299,21 @@ static double beta_of(int precision, int slices = 0)
 // measured per kernel on GB300 at 2070 MHz.  The
 // instruction roof t * SMs * clock / cycles per output caps the paper's
 // tensor-core roof (Eq. 12) for the dispatcher.
+//
+// For 2-D FP32 grids the constants were measured on the line-form kernels and on
+// the tiled CUDA-core sweep.  The block-form kernels (k_wide.cu) and the marching
+// kernel run faster than these roofs: Box-2D2R on 16384^2 FP16 t = 4 1201 predicted,
+// 2170 GStencil/s measured; native t = 1 490 and 703.  They rank (path, t) in the
+// order of the earlier kernels, which is conservative in t: on 6000 x 5000 the t they
+// choose is the fastest for r = 1 and 2 in the FP16 and BF16 forms, and up to 1.8 times
+// slower than t = 4 for TF32, 2.0 for TF32x3 and 1.7 for radius 3 (stencil_plan_autotune
+// measures instead).  k_split.cu issues an MMA in ~50 cycles now, not 90.
 // ---------------------------------------------------------------------------
 constexpr double kMmaCycles = 90.0;        // per tcgen05.mma, M = 128, N <= ~176
-constexpr double kWorkerTf32 = 1.30;       // tc2d_ws TF32: in-place rounding, staging, epilogue
-constexpr double kWorkerTf32x3 = 1.65;     // tc2d_ws TF32x3: + the lo split
-constexpr double kWorkerWide = 0.45;       // tc2d_wide, one product: loads, conversion, epilogue (added to the MMAs)
-constexpr double kWorkerWideSplit = 0.28;  // tc2d_wide, three products (128-row tiles, one or two buffers)
+constexpr double kWorkerTf32 = 1.30;       // line form TF32: in-place rounding, staging, epilogue
+constexpr double kWorkerTf32x3 = 1.65;     // line form TF32x3: + the lo split
+constexpr double kWorkerWide = 0.45;       // line form FP16: loads, conversion, epilogue (added to the MMAs)
+constexpr double kWorkerWideSplit = 0.28;  // line form, three products (128-row tiles, one or two buffers)
 constexpr double kWorkerWide3 = 0.78;      // tc3d_wide, 128-row tiles: plane staging, strips, epilogue, runs
 constexpr double kWorkerSplit = 4.06;      // tc2d_split: FP64 load, exponent, digit cut, recombination
 // sptc2d_sweep issues warp-level mma.sp between its staging and epilogue
@@ -364,7 +373,7 @@ static double tc_instr_gstencils(const Plan &p, int prec, int path, int t)
     } else if (p.dtype == STENCIL_F32 &&
                (prec == STENCIL_PREC_F16 || prec == STENCIL_PREC_F16X3 || prec == STENCIL_PREC_BF16X3) &&
                tc_wide_nrows(r, t, prec != STENCIL_PREC_F16) > 0) {
-        // tc2d_wide: per tile of 128 columns x nr rows, one MMA (M = 128,
+        // line form: per tile of 128 columns x nr rows, one MMA (M = 128,
         // N = nr, K = 16) per (line, K block) and product, each costing
         // max(kMmaCycles, its arithmetic at 4096 FP16 MACs per cycle)
         const int nr = tc_wide_nrows(r, t, prec != STENCIL_PREC_F16);
@@ -559,7 +568,9 @@ stencil_status dispatch(Plan *p)
     // kernel runs it.  The ranking's instruction roofs describe the line-form
     // kernels, among which the sparse one led from t = 3; the block form
     // (k_wide.cu) is faster than the sparse kernel at every t and radius
-    // measured.  The two forms round the same operands to TF32, so the choice
+    // measured (GStencil/s on 4001 x 3003, dense and sparse at t = 1, 2, 4: Box-2D1R
+    // 385 640 1062 and 192 335 551, Box-2D2R 268 469 855 and 177 282 346, Star-2D3R
+    // 262 521 638 and 168 249 176).  The two forms round the same operands to TF32, so the choice
     // changes results by FP32 accumulation order only, which a different t
     // would not.
     if (pick->path == STENCIL_PATH_SPARSE_TENSOR_CORE && p->req_path == STENCIL_PATH_AUTO) {

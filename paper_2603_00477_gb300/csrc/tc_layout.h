@@ -1,6 +1,10 @@
-// tc_layout.h -- geometry of the tensor-core (Toeplitz) formulation, shared by
-// the dispatcher (which reports the sparsity factor S, paper Sec. 2.2.2) and
-// the launchers (which issue exactly the MMAs counted here).
+// tc_layout.h -- geometry of the tensor-core (Toeplitz) formulation.  The line
+// form below is the reference layout: stencil_plan_tc_layout exports it, the
+// sparsity factor S (paper Sec. 2.2.2) and the dispatcher's roofs are computed from
+// it, and the FP64 MMA kernel (k_tc.cu), the exact-split kernel (k_split.cu) and the
+// 3-D kernel (k_wide3d.cu) issue exactly the MMAs counted here.  The 2-D FP32 kernels
+// (k_wide.cu) issue the denser block form (BlockTile, further down): fewer MMAs for
+// the same products.
 //
 // The t-step composite kernel w^(t) of radius R = t*r is applied as a sum
 // over its rows ("lines"; in 3-D over (plane,row) pairs): for line a,
@@ -65,8 +69,7 @@ inline TcLines tc_lines_2d(int shape, int r, int t, int n_tile, int k_inst)
     return L;
 }
 
-// MMA N (output columns per Toeplitz block) of the warp-specialised TF32 /
-// TF32x3 kernel: the widest of 32, 16, 8 whose operands fit in 227 KB of
+// MMA N (output columns per Toeplitz block) of the TF32 / TF32x3 line form: the widest of 32, 16, 8 whose operands fit in 227 KB of
 // shared memory -- B blocks (x2 split) plus double-buffered A tiles (hi, and
 // lo when split) of 128 + 2R rows (rounded up to 8) by (NACC-1)*N + kext columns.
 inline int tc_ws_ntile(int shape, int r, int t, bool split)
@@ -140,10 +143,14 @@ inline BlockTile tc_block_geom(int R, bool tf32, bool split, int gn, int hx, int
 // The tile of a grid with ny interior rows and ex stored columns on `sms` SMs:
 // the least (rounds of CTAs) x (cycles per tile) over gn = 32 .. 4, hx = 2 or 1
 // and two operand buffers or one (one only where no two fit).  Cycles per
-// tile, measured: an MMA takes N / 2 = 4 gn cycles, at least 50; staging 1.0 per
+// tile: an MMA takes N / 2 = 4 gn cycles, at least 50 (measured); staging 1.0 per
 // 16 bytes; HBM 1.15 x 8 bytes per output at 21.5 bytes per cycle and SM.  They
 // overlap with two operand buffers; with one, staging and MMAs take turns.
 // 2000 cycles per tile do not overlap (first loads, scale exchange, hand-over).
+// The terms rank tiles; their sum is no prediction: fitted to FP16 t = 4 on 16384^2
+// (16k cycles per 256 x 128 tile, 18k measured), it gives 9k for the TF32 t = 7 tile on
+// 10240^2 that takes 13k, and half of what a sweep of a few rounds takes, whose
+// strips and first loads it leaves out.
 inline BlockTile tc_block_tile(int R, bool tf32, bool split, int64_t ny, int64_t ex, int sms)
 {
     BlockTile best;
