@@ -228,12 +228,18 @@ def traffic_record(kernel_key):
 
 
 
-def kernel_name(info: dict, d: int, dtype: str, shape: str = "box", r: int = 1) -> str:
+def kernel_name(info: dict, d: int, dtype: str, shape: str = "box", r: int = 1, dims=None) -> str:
     """The sweep kernel a plan launches, from its stencil, path, precision,
-    tile and t (the rules of the library's launchers)."""
+    default tile, t and (Box-2D3R FP32 at t = 1) extents (the rules of the
+    library's launchers)."""
     if info["path"] == 1:
         if d == 2:
-            return "cu2d_sweep"
+            # FP32, default tile: the marching kernel where it has the depth, but tiles for Box-2D3R at t = 1
+            # on grids that the tile divides
+            march = dtype == "f32" and r <= 3 and (info["t"] == 1 or (info["t"] == 2 and not (shape == "box" and r == 3)))
+            if march and shape == "box" and r == 3 and dims and dims[0] * dims[1] <= 6000000:
+                march = dims[0] % info["tile"][1] != 0 or dims[1] % info["tile"][2] != 0
+            return "cu2d_march" if march else "cu2d_sweep"
         if info["t"] != 1:
             return "cu3d_sweep"
         # FP32 star r <= 3 and box r = 1 take the rotating kernel
@@ -865,7 +871,7 @@ def main():
     avg_launch_s = ms / 1e3 / sweep_launches
     K = info["K"]
     D = 8 if cfg["dtype"] == "f64" else 4
-    kernel = kernel_name(info, cfg["d"], cfg["dtype"], cfg["shape"], cfg["r"])
+    kernel = kernel_name(info, cfg["d"], cfg["dtype"], cfg["shape"], cfg["r"], cfg["dims"])
     kernel_key = f"{kernel}:{args.config}:{info['path_name']}:t{t}"
     traffic = traffic_record(kernel_key)
     if info["memory_bound"]:
