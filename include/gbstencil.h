@@ -97,8 +97,8 @@ typedef enum {
  * takes K = 16 per instruction against TF32's 8.  3-D grids take the
  * tensor-core path only as FP32 in the F16 form at t = 1 (box r <= 2, star
  * r <= 3; a power-of-two scale per staged plane tile that leaves its largest
- * |x| in [2^6, 2^15), so that values down to 2^-20 of it keep 11 bits).  ANY: the dispatcher
- * may pick any form the grid type allows. */
+ * |x| in [2^6, 2^15), so that values down to 2^-20 of it keep 11 bits).
+ * ANY: the dispatcher may pick any form the grid type allows. */
 typedef enum {
     STENCIL_PREC_NATIVE = 0,
     STENCIL_PREC_TF32 = 1,

@@ -29,9 +29,9 @@ inline bool next_sweep_early(bool f64, int r, int t, int64_t tiles, int64_t resi
 }
 
 // Items of the busiest SM when persistent CTAs, `occ` resident per SM, work off `items`.  Up to one wave the CTAs
-// are spread evenly; beyond it those that take one item more share an SM as soon as they are more than ~4/5 of
-// the SMs (the block scheduler fills the smaller GPCs twice before the larger ones once): 448 items on 304 CTAs
-// are four on some SMs, not three.
+// are spread evenly; beyond it those that take one item more were measured to share an SM as soon as they are more
+// than ~4/5 of the SMs (as if smaller GPCs were filled twice before larger ones once): 448 items on 304 CTAs
+// take as long as four on some SMs, not three.
 inline int64_t busiest_items(int64_t items, int occ, int sms)
 {
     const int64_t wave = (int64_t)occ * sms, full = items / wave, rest = items % wave;
