@@ -143,7 +143,7 @@ typedef struct {
     int scenario;         /* 1..4 (Sec. 4.1) of CU vs TC at this t           */
     int memory_bound;     /* 1 if the chosen path is below its ridge         */
     /* The dispatcher's model.  Its instruction roofs for 2-D FP32 grids
-     * were measured on earlier kernels; the present ones run up to about twice
+     * were measured on earlier kernels; the present ones run up to three times
      * as fast (stencil_plan_autotune measures). */
     double predicted_gstencils;    /* point-updates/s / 1e9 at the roof      */
     double predicted_cu_gstencils; /* CU path at this t                      */

@@ -303,7 +303,7 @@ static double beta_of(int precision, int slices = 0)
 // For 2-D FP32 grids the constants were measured on the line-form kernels and on
 // the tiled CUDA-core sweep.  The block-form kernels (k_wide.cu) and the marching
 // kernel run faster than these roofs: Box-2D2R on 16384^2 FP16 t = 4 1201 predicted,
-// 2170 GStencil/s measured; native t = 1 490 and 703.  They rank (path, t) in the
+// 2189 GStencil/s measured; TF32 t = 4 562 and 1667; native t = 1 490 and 703.  They rank (path, t) in the
 // order of the earlier kernels, which is conservative in t: on 6000 x 5000 the t they
 // choose is the fastest for r = 1 and 2 in the FP16 and BF16 forms, and up to 1.8 times
 // slower than t = 4 for TF32, 2.0 for TF32x3 and 1.7 for radius 3 (stencil_plan_autotune
